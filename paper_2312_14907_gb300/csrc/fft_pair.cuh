@@ -18,8 +18,6 @@
 
 namespace mpbp {
 
-MPBP_DI cf cadd(cf a, cf b) { return cf{a.x + b.x, a.y + b.y}; }
-MPBP_DI cf csub(cf a, cf b) { return cf{a.x - b.x, a.y - b.y}; }
 MPBP_DI cf csel(bool c, cf a, cf b) { return cf{c ? a.x : b.x, c ? a.y : b.y}; }
 
 template <int L, typename Xchg>
