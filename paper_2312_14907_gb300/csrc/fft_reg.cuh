@@ -152,21 +152,28 @@ MPBP_DI void bfly(cf& a, cf& b) {
   }
 }
 
+// Butterflies b in [B0, B1) of stage S (span 2^S) of fft_line<L> below, for
+// callers that interleave the stages with loads and stores: stages 0..S of
+// the natural indices n = c mod L / 2^(S+1) touch those indices alone, and are
+// the butterflies [2^S c', 2^S (c' + 1)), c' the bit reversal of c.
+template <int L, int S, int B0, int B1>
+MPBP_DI void fft_stage(cf (&x)[L]) {
+  constexpr int span = 1 << S;
+  sfor<B0, B1>([&](auto b_) {
+    constexpr int b = decltype(b_)::value;
+    constexpr int grp = b / span, k = b % span;
+    constexpr int i0 = ct::brev<L>(grp * 2 * span + k);
+    constexpr int i1 = ct::brev<L>(grp * 2 * span + k + span);
+    bfly<k, 2 * span>(x[i0], x[i1]);
+  });
+}
+
 // In-place L-point forward DFT of x[0..L) (natural order in).  Decimation in
 // time on the bit-reversed view of the array: afterwards X[k] = x[brev(k)].
 template <int L>
 MPBP_DI void fft_line(cf (&x)[L]) {
   constexpr int LOG = ct::ilog2(L);
-  sfor<0, LOG>([&](auto s_) {
-    constexpr int span = 1 << decltype(s_)::value;
-    sfor<0, L / 2>([&](auto b_) {
-      constexpr int b = decltype(b_)::value;
-      constexpr int grp = b / span, k = b % span;
-      constexpr int i0 = ct::brev<L>(grp * 2 * span + k);
-      constexpr int i1 = ct::brev<L>(grp * 2 * span + k + span);
-      bfly<k, 2 * span>(x[i0], x[i1]);
-    });
-  });
+  sfor<0, LOG>([&](auto s_) { fft_stage<L, decltype(s_)::value, 0, L / 2>(x); });
 }
 
 // multiply by a compile-time twiddle W_N^K

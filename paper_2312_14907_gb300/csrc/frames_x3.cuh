@@ -23,6 +23,17 @@
 // The twiddles W^(h k'), h = 1..3, and W^(m' c_r), m' = 1..7, are formed once
 // per block into a 1.7 KB shared table.
 //
+// What bounds it: per frame the FP32 pipes work about 11.7 K clocks and
+// shared memory moves 1.3 MB (10.4 K clocks at 128 B); between the barriers
+// of the exchanges the two overlap only in part (20.7 K clocks in all).  So
+// the loads of a phase stand ahead of its first transforms and the stores
+// behind the last ones they need, not behind all: the 32-point transforms
+// run by n mod 4 while the patch and the probe values still arrive, and each
+// layout's results are stored as its last stage yields them (1024^2 workload,
+// 87,846 frames: 6.31 -> 6.01 ms a call; splitting the "all read" barriers
+// into an arrival and a wait cost 0.16 ms of it, passing the loads from warp
+// group to warp group 0.8 ms).
+//
 // Gradient accumulation (A7).  A block takes a contiguous range of the
 // frames in the order it is given; the host orders them by peak, scan column
 // and scan row, so that a block's consecutive frames mostly share their
@@ -270,48 +281,94 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
                       uint32_t ta, const X3Tables& tab, X3Win& win) {
   using C = X3Cfg;
   constexpr int M = C::M, PW = C::PW;
-  // the probe values of A2 load from tensor memory while the inputs land
-  uint32_t w[4][16];
-  sfor<0, 4>([&](auto c_) { tmem_ld16(tp + 16 * decltype(c_)::value, w[decltype(c_)::value]); });
+  // ---- A2 + the 32-point transforms over n (L1), by n mod 4: a chunk's probe
+  // values come from tensor memory (the first while the inputs land) and its
+  // patch values from shared memory ahead of the chunk before
+  uint32_t w[2][16];
+  tmem_ld16(tp, w[0]);
+  bool ok = true;
   if constexpr (TMA) {
-    bs.ok = bulk_wait(bs.bar, bs.parity);
+    ok = bulk_wait_thread(bs.bar, bs.parity);   // the block agrees on it below
     bs.parity ^= 1u;
-    if (!bs.ok) {
-      tmem_wait_ld();
-      return;
-    }
   } else {
     cp_async_wait_all();
     __syncthreads();
   }
-  tmem_fence_after_sync();   // the previous frame's window updates
-  const int dlt = TMA ? (cur.s.y & 1) : 0;   // a tile starts at an even column
-
-  // ---- A2 + the 32-point transforms over n (L1)
-  cf v[32];
-  tmem_wait_ld();
-  sfor<0, 32>([&](auto n_) {
-    constexpr int n = decltype(n_)::value;
-    const cf pv = cf{__uint_as_float(w[n % 4][2 * (n / 4)]), __uint_as_float(w[n % 4][2 * (n / 4) + 1])};
-    v[n] = cmul(pv, buf[(4 * n + r.h) * PW + r.c + dlt]);
+  const cf* const patch = buf + r.h * PW + r.c + (TMA ? (cur.s.y & 1) : 0);   // a tile starts at an even column
+  cf v[32], o[8];
+  sfor<0, 8>([&](auto m_) { o[decltype(m_)::value] = patch[16 * decltype(m_)::value * PW]; });
+  sfor<0, 4>([&](auto c_) {
+    constexpr int c = decltype(c_)::value, cb = ct::brev<4>(c);
+    tmem_wait_ld();
+    if constexpr (c < 3) tmem_ld16(tp + 16 * (c + 1), w[(c + 1) & 1]);
+    sfor<0, 8>([&](auto m_) {
+      constexpr int m = decltype(m_)::value;
+      v[4 * m + c] =
+          cmul(cf{__uint_as_float(w[c & 1][2 * m]), __uint_as_float(w[c & 1][2 * m + 1])}, o[m]);
+    });
+    if constexpr (c < 3)
+      sfor<0, 8>([&](auto m_) {
+        constexpr int m = decltype(m_)::value;
+        o[m] = patch[4 * (4 * m + c + 1) * PW];
+      });
+    fft_stage<32, 0, 4 * cb, 4 * cb + 4>(v);
+    fft_stage<32, 1, 4 * cb, 4 * cb + 4>(v);
+    fft_stage<32, 2, 4 * cb, 4 * cb + 4>(v);
   });
-  fft_line<32>(v);   // Y(h, k', c) in slot brev(k')
   __syncthreads();   // the patch reads are done
-  sfor<0, 32>([&](auto k_) {
+  tmem_fence_after_sync();   // the previous frame's window updates
+  sfor<0, 8>([&](auto k_) {
     constexpr int k = decltype(k_)::value;
-    buf[x3_a(r.h, k, r.c)] = v[ct::brev<32>(k)];
+    fft_stage<32, 3, k, k + 1>(v);
+    fft_stage<32, 3, k + 8, k + 9>(v);
+    fft_stage<32, 4, k, k + 1>(v);
+    fft_stage<32, 4, k + 8, k + 9>(v);
+    sfor<0, 4>([&](auto t_) {
+      constexpr int kp = k + 8 * decltype(t_)::value;
+      buf[x3_a(r.h, kp, r.c)] = v[ct::brev<32>(kp)];   // Y(h, k', c)
+    });
   });
+  if constexpr (!LOSS) {
+    // the window moves to this frame's rows: rows that leave it go out
+    // (here, where few registers are live, beside other warps' stores)
+    if (cur.valid) {
+      const bool slide = win.ok && cur.mpk == win.mpk && cur.s.y == win.y && cur.s.x >= win.x &&
+                         cur.s.x - win.x < X3Cfg::M;
+      const int dd = slide ? cur.s.x - win.x : X3Cfg::M;
+      if (win.ok) x3_flush<DET>(p, r, win, win.x, dd, ta, true);
+      // a new strip starts the block's next piece (the host splits them there)
+      const bool strip = !win.ok || cur.mpk != win.mpk || cur.s.y != win.y;
+      int wlo = win.wlo, whi = win.whi;
+      if (win.ok && dd > 0) {
+        wlo = min(wlo, win.x);
+        whi = max(whi, win.x + dd);
+      }
+      if (strip) {
+        wlo = INT_MAX;
+        whi = INT_MIN;
+      }
+      win = X3Win{true, cur.mpk, cur.s.y, cur.s.x, win.piece + (strip ? 1 : 0), wlo, whi};
+    }
+    tmem_wait_st();
+    tmem_fence_before_sync();   // the slots the window left are clear
+  }
   cf x[32];
   {
   X3Tw tw;
   x3_twiddles(tab, r, tw);   // the table is constant: read ahead of the barrier
-  __syncthreads();
+  if constexpr (TMA) {
+    bs.ok = __syncthreads_and((int)ok) != 0;
+    if (!bs.ok) return;
+  } else {
+    __syncthreads();
+  }
+  if constexpr (!LOSS) tmem_fence_after_sync();
 
   // ---- L2: twiddle, 4-point over h, 8-point over c_a, twiddle
-  sfor<0, 4>([&](auto h_) {
-    constexpr int hh = decltype(h_)::value;
-    sfor<0, 8>([&](auto a_) {
-      constexpr int ca = decltype(a_)::value;
+  sfor<0, 8>([&](auto a_) {
+    constexpr int ca = decltype(a_)::value;
+    sfor<0, 4>([&](auto h_) {
+      constexpr int hh = decltype(h_)::value;
       x[hh * 8 + ca] = buf[x3_a(hh, r.kp, r.cr + 16 * ca)];
     });
   });
@@ -329,45 +386,27 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
       x[kk * 8 + ca] = t4[ct::brev<4>(kk)];   // x[8 k'' + c_a]
     });
   });
+  __syncthreads();   // every layout-A read is done
   sfor<0, 4>([&](auto k_) {
     constexpr int kk = decltype(k_)::value;
     cf t8[8];
     sfor<0, 8>([&](auto a_) { t8[decltype(a_)::value] = x[kk * 8 + decltype(a_)::value]; });
     fft_line<8>(t8);
-    x[kk * 8] = t8[0];
-    sfor<1, 8>([&](auto m_) {
+    sfor<0, 8>([&](auto m_) {
       constexpr int mp = decltype(m_)::value;
-      x[kk * 8 + mp] = cmul(t8[ct::brev<8>(mp)], tw.um[mp]);   // x[8 k'' + m']
+      const cf z = t8[ct::brev<8>(mp)];
+      if constexpr (mp == 0) buf[x3_b(0, r.kp + 32 * kk, r.cr)] = z;
+      else buf[x3_b(mp, r.kp + 32 * kk, r.cr)] = cmul(z, tw.um[mp]);
     });
   });
   }
-  __syncthreads();   // every layout-A read is done
-  sfor<0, 4>([&](auto k_) {
-    constexpr int kk = decltype(k_)::value;
-    sfor<0, 8>([&](auto m_) {
-      constexpr int mp = decltype(m_)::value;
-      buf[x3_b(mp, r.kp + 32 * kk, r.cr)] = x[kk * 8 + mp];
-    });
-  });
   __syncthreads();
 
-  // ---- L3: 16-point over c_r; A4 on row q0
-  sfor<0, 2>([&](auto m_) {
-    constexpr int mr = decltype(m_)::value;
-    sfor<0, 16>([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      v[mr * 16 + i] = buf[x3_b(r.mt + 4 * mr, r.q0, i)];
-    });
-  });
-  sfor<0, 2>([&](auto m_) {
-    constexpr int mr = decltype(m_)::value;
-    cf t16[16];
-    sfor<0, 16>([&](auto i_) { t16[decltype(i_)::value] = v[mr * 16 + decltype(i_)::value]; });
-    fft_line<16>(t16);
-    sfor<0, 16>([&](auto i_) {
-      constexpr int mm = decltype(i_)::value;
-      v[mr * 16 + mm] = t16[ct::brev<16>(mm)];   // Psi(q0, m' + 8 m'') at v[16 m_r + m'']
-    });
+  // ---- L3: 16-point over c_r; A4 on row q0; A5: Z = F conj(chi), 16-point
+  // over m''
+  sfor<0, 32>([&](auto i_) {
+    constexpr int i = decltype(i_)::value;
+    v[i] = buf[x3_b(r.mt + 4 * (i / 16), r.q0, i % 16)];
   });
   float fl = 0.0f;
   // BG: the background b of Eq. 2 (a kernel of its own, so that the common
@@ -375,12 +414,23 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
   const float* bg = BG ? p.bgT + (long long)cur.f * M * M : nullptr;
   sfor<0, 2>([&](auto m_) {
     constexpr int mr = decltype(m_)::value;
+    cf t16[16], z16[16];
+    sfor<0, 16>([&](auto i_) { t16[decltype(i_)::value] = v[mr * 16 + decltype(i_)::value]; });
+    fft_line<16>(t16);   // Psi(q0, m' + 8 m'') in slot brev(m'')
     sfor<0, 16>([&](auto i_) {
       constexpr int mm = decltype(i_)::value;
       const int q1 = r.mt + 4 * mr + 8 * mm;
       const float bv = BG ? bg[q1 * M + r.q0] : 0.0f;
-      v[mr * 16 + mm] = residual(v[mr * 16 + mm], abuf[q1 * M + r.q0], bv, fl);
+      z16[mm] = residual(t16[ct::brev<16>(mm)], abuf[q1 * M + r.q0], bv, fl);
     });
+    if constexpr (!LOSS) {
+      fft_line<16>(z16);   // T(m', kr) in slot brev(kr)
+      if constexpr (mr == 0) __syncthreads();   // every layout-B read is done
+      sfor<0, 16>([&](auto i_) {
+        constexpr int kr = decltype(i_)::value;
+        buf[x3_b(r.mt + 4 * mr, r.q0, kr)] = z16[ct::brev<16>(kr)];
+      });
+    }
   });
   add_loss(cur.valid ? 0.5f * fl : 0.0f);
   if constexpr (LOSS) {
@@ -389,41 +439,25 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
     if constexpr (!TMA) cp_async_commit();
     return;
   }
-
-  // ---- A5: Z = F conj(chi), L3: 16-point over m''
-  sfor<0, 2>([&](auto m_) {
-    constexpr int mr = decltype(m_)::value;
-    cf t16[16];
-    sfor<0, 16>([&](auto i_) { t16[decltype(i_)::value] = v[mr * 16 + decltype(i_)::value]; });
-    fft_line<16>(t16);   // T(m', kr) in slot brev(kr)
-    sfor<0, 16>([&](auto i_) {
-      constexpr int kr = decltype(i_)::value;
-      v[mr * 16 + kr] = t16[ct::brev<16>(kr)];
-    });
-  });
-  __syncthreads();   // every layout-B read is done
-  sfor<0, 2>([&](auto m_) {
-    constexpr int mr = decltype(m_)::value;
-    sfor<0, 16>([&](auto i_) {
-      constexpr int kr = decltype(i_)::value;
-      buf[x3_b(r.mt + 4 * mr, r.q0, kr)] = v[mr * 16 + kr];
-    });
-  });
-  // the residual's reads of the sqrt(y) buffer are behind the barrier above:
-  // the next frame's tile can land there now
-  if constexpr (TMA) x3_fetch_amp_tma(p, r, nxt, abuf, bs, tm);
   X3Tw tw;
   x3_twiddles(tab, r, tw);
   __syncthreads();
+  // every thread is past the residual, which read the sqrt(y) buffer: the
+  // next frame's tile can land there now
+  if constexpr (TMA) x3_fetch_amp_tma(p, r, nxt, abuf, bs, tm);
 
   // ---- L2: twiddle, 8-point over m', 4-point over k'', twiddle
+  sfor<0, 32>([&](auto i_) {
+    constexpr int i = decltype(i_)::value;
+    x[i] = buf[x3_b(i % 8, r.kp + 32 * (i / 8), r.cr)];
+  });
   sfor<0, 4>([&](auto k_) {
     constexpr int kk = decltype(k_)::value;
     cf t8[8];
-    t8[0] = buf[x3_b(0, r.kp + 32 * kk, r.cr)];
+    t8[0] = x[kk * 8];
     sfor<1, 8>([&](auto m_) {
       constexpr int mp = decltype(m_)::value;
-      t8[mp] = cmul(buf[x3_b(mp, r.kp + 32 * kk, r.cr)], tw.um[mp]);
+      t8[mp] = cmul(x[kk * 8 + mp], tw.um[mp]);
     });
     fft_line<8>(t8);
     sfor<0, 8>([&](auto a_) {
@@ -431,67 +465,34 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
       x[kk * 8 + ka] = t8[ct::brev<8>(ka)];   // x[8 k'' + k_a]
     });
   });
+  __syncthreads();   // every layout-B read is done
   sfor<0, 8>([&](auto a_) {
     constexpr int ka = decltype(a_)::value;
     cf t4[4];
     sfor<0, 4>([&](auto k_) { t4[decltype(k_)::value] = x[decltype(k_)::value * 8 + ka]; });
     fft_line<4>(t4);
-    x[ka] = t4[0];
-    sfor<1, 4>([&](auto h_) {
+    sfor<0, 4>([&](auto h_) {
       constexpr int hh = decltype(h_)::value;
-      x[hh * 8 + ka] = cmul(t4[ct::brev<4>(hh)], tw.th[hh]);   // x[8 h' + k_a]
-    });
-  });
-  __syncthreads();   // every layout-B read is done
-  sfor<0, 4>([&](auto h_) {
-    constexpr int hh = decltype(h_)::value;
-    sfor<0, 8>([&](auto a_) {
-      constexpr int ka = decltype(a_)::value;
-      buf[x3_a(hh, r.kp, r.cr + 16 * ka)] = x[hh * 8 + ka];
+      const cf z = t4[ct::brev<4>(hh)];
+      if constexpr (hh == 0) buf[x3_a(0, r.kp, r.cr + 16 * ka)] = z;
+      else buf[x3_a(hh, r.kp, r.cr + 16 * ka)] = cmul(z, tw.th[hh]);
     });
   });
   __syncthreads();
 
   // ---- L1: 32-point over k'; A6 + A7
-  sfor<0, 32>([&](auto k_) {
-    constexpr int k = decltype(k_)::value;
-    v[k] = buf[x3_a(r.h, k, r.c)];
-  });
-  // the window moves to this frame's rows: rows that leave it go out
-  if (cur.valid) {
-    const bool slide = win.ok && cur.mpk == win.mpk && cur.s.y == win.y && cur.s.x >= win.x &&
-                       cur.s.x - win.x < X3Cfg::M;
-    const int dd = slide ? cur.s.x - win.x : X3Cfg::M;
-    if (win.ok) x3_flush<DET>(p, r, win, win.x, dd, ta, true);
-    // a new strip starts the block's next piece (the host splits them there)
-    const bool strip = !win.ok || cur.mpk != win.mpk || cur.s.y != win.y;
-    int wlo = win.wlo, whi = win.whi;
-    if (win.ok && dd > 0) {
-      wlo = min(wlo, win.x);
-      whi = max(whi, win.x + dd);
-    }
-    if (strip) {
-      wlo = INT_MAX;
-      whi = INT_MIN;
-    }
-    win = X3Win{true, cur.mpk, cur.s.y, cur.s.x, win.piece + (strip ? 1 : 0), wlo, whi};
-  }
-  tmem_wait_st();
-  tmem_fence_before_sync();
-  __syncthreads();   // both buffers are free; the slots the window left are clear
-  tmem_fence_after_sync();
-  if constexpr (TMA) {
-    x3_fetch_patch_tma(r, nxt, buf, bs, tm);
-  } else {
-    x3_fetch<false>(p, r, nxt, buf, abuf, bs, tm);
-    cp_async_commit();
-  }
-  if (!cur.valid) return;
   // the 32-point transform over k' split by frequency, n = 4 m + r:
   //   Z(n) = sum_j W8^(j m) [W32^(j r) sum_s W4^(s r) v(j + 8 s)],
   // a radix-4 step, then one 8-point transform per r, whose outputs are
   // multiplied by the probe (A6) and added into the window's slots of rows
   // s.x + h + 4 n
+  sfor<0, 8>([&](auto j_) {
+    constexpr int j = decltype(j_)::value;
+    sfor<0, 4>([&](auto t_) {
+      constexpr int k = j + 8 * decltype(t_)::value;
+      v[k] = buf[x3_a(r.h, k, r.c)];
+    });
+  });
   sfor<0, 8>([&](auto j_) {
     constexpr int j = decltype(j_)::value;
     cf t4[4] = {v[j], v[j + 8], v[j + 16], v[j + 24]};
@@ -501,14 +502,22 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
       v[j + 8 * rr] = twmul<j * rr, 32>(t4[ct::brev<4>(rr)]);   // u_r(j) at v[j + 8 r]
     });
   });
+  __syncthreads();   // both buffers are free
+  if constexpr (TMA) {
+    x3_fetch_patch_tma(r, nxt, buf, bs, tm);
+  } else {
+    x3_fetch<false>(p, r, nxt, buf, abuf, bs, tm);
+    cp_async_commit();
+  }
+  if (!cur.valid) return;
   const int b0 = cur.s.x + r.h;   // row of n = 0
   sfor<0, 4>([&](auto r_) {
     constexpr int rr = decltype(r_)::value;
-    uint32_t pw[16], o[8][2];
+    uint32_t pw[16], ow[8][2];
     tmem_ld16(tp + 16 * rr, pw);   // P at n = 4 m + r, m = 0..7
     sfor<0, 8>([&](auto m_) {
       constexpr int m = decltype(m_)::value;
-      tmem_ld2(ta + 2u * (uint32_t)((b0 + 4 * (4 * m + rr)) & 127), o[m]);
+      tmem_ld2(ta + 2u * (uint32_t)((b0 + 4 * (4 * m + rr)) & 127), ow[m]);
     });
     cf t8[8];
     sfor<0, 8>([&](auto j_) { t8[decltype(j_)::value] = v[decltype(j_)::value + 8 * rr]; });
@@ -518,8 +527,8 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
       constexpr int m = decltype(m_)::value;
       const cf pv = cf{__uint_as_float(pw[2 * m]), __uint_as_float(pw[2 * m + 1])};
       const cf z = t8[ct::brev<8>(m)];
-      const float gx = fmaf(pv.x, z.x, fmaf(-pv.y, z.y, __uint_as_float(o[m][0])));
-      const float gy = fmaf(pv.x, z.y, fmaf(pv.y, z.x, __uint_as_float(o[m][1])));
+      const float gx = fmaf(pv.x, z.x, fmaf(-pv.y, z.y, __uint_as_float(ow[m][0])));
+      const float gy = fmaf(pv.x, z.y, fmaf(pv.y, z.x, __uint_as_float(ow[m][1])));
       tmem_st2(ta + 2u * (uint32_t)((b0 + 4 * (4 * m + rr)) & 127), __float_as_uint(gx), __float_as_uint(gy));
     });
   });
