@@ -83,7 +83,7 @@ struct FramesKernel<M, false> {
   static KernelShape grad(bool, bool = false, int = 0, bool = false, bool = false) {
     return {frames_t1<M, false>, C::T, C::SMEM};
   }
-  static KernelShape fwd(bool) { return {frames_t1<M, true>, C::T, C::SMEM}; }
+  static KernelShape fwd(bool, bool = false) { return {frames_t1<M, true>, C::T, C::SMEM}; }
   static KernelShape loss(bool, bool = false, int = 0, bool = false) {
     return {frames_t1<M, false, true>, C::T, C::SMEM};
   }
@@ -97,7 +97,7 @@ struct FramesKernel<M, true> {
   using C = T2Cfg<M>;
   static constexpr bool kQuads = UseQuads<M>::value;
   static constexpr int NG = 1;
-  static constexpr int kTileFwd = C::PW;
+  static constexpr int kTileFwd = kQuads ? X3Cfg::PW : C::PW;
   static constexpr int kTileGrad = kQuads ? T4Cfg<M>::PW : (C::SWZ ? 0 : C::PW);
   // tpr: the probe stays in tensor memory (four threads per line; probes
   // shared by the frames of a peak)
@@ -127,9 +127,19 @@ struct FramesKernel<M, true> {
                  : KernelShape{frames_t2<M, false>, C::T, C::SMEM};
     }
   }
-  static KernelShape fwd(bool tma) {
-    return tma ? KernelShape{frames_t2<M, true, false, true>, C::T, C::SMEM_TMA}
-               : KernelShape{frames_t2<M, true>, C::T, C::SMEM};
+  // M = 128: the exchange kernel's first half (14,884 frames of a 512^2 object:
+  // 612 us a call; the thread-pair layout with its 64 values a thread 945)
+  static KernelShape fwd(bool tma, bool bg = false) {
+    if constexpr (kQuads) {
+      if (bg)
+        return {tma ? frames_x3<true, false, true, false, true> : frames_x3<false, false, true, false, true>, X3Cfg::T,
+                X3Cfg::SMEM_FWD};
+      return {tma ? frames_x3<true, false, false, false, true> : frames_x3<false, false, false, false, true>, X3Cfg::T,
+              X3Cfg::SMEM_FWD};
+    } else {
+      return tma ? KernelShape{frames_t2<M, true, false, true>, C::T, C::SMEM_TMA}
+                 : KernelShape{frames_t2<M, true>, C::T, C::SMEM};
+    }
   }
   // the loss alone, in the gradient kernel's layout (same tile width)
   static KernelShape loss(bool tma, bool tpr = false, int layout = kLayoutDefault, bool bg = false) {
@@ -174,7 +184,7 @@ bool frames_prepare_impl(FrameKernelInfo* info) {
   using K = FramesKernel<M>;
   bool ok = true;
   for (int t = 0; t < 32; ++t)
-    ok = set_smem(K::grad(t & 1, (t >> 1) & 1, (t >> 2) & 1, (t >> 3) & 1, t >> 4)) && set_smem(K::fwd(t & 1)) &&
+    ok = set_smem(K::grad(t & 1, (t >> 1) & 1, (t >> 2) & 1, (t >> 3) & 1, t >> 4)) && set_smem(K::fwd(t & 1, (t >> 1) & 1)) &&
          set_smem(K::loss(t & 1, (t >> 1) & 1, (t >> 2) & 1, (t >> 3) & 1)) && ok;
   if (K::kRaw) ok = set_smem(K::raw(false)) && set_smem(K::raw(true)) && ok;
   if (K::kRaw16) ok = set_smem(K::raw(true, true)) && ok;
@@ -202,7 +212,7 @@ cudaError_t frames_launch_impl(const FrameArgs& a, int grid, bool forward, cudaS
   using K = FramesKernel<M>;
   static const TmaMap kNone{};
   const bool tile = tm != nullptr && (forward ? K::kTileFwd : K::kTileGrad) > 0;
-  const KernelShape k = forward ? K::fwd(tile)
+  const KernelShape k = forward ? K::fwd(tile, a.bgT != nullptr)
                                 : K::grad(tile, a.probe_stride >= 0, layout, a.bgT != nullptr, a.det != nullptr);
   k.fn<<<grid, k.threads, k.smem, s>>>(a, tile ? *tm : kNone);
   return cudaGetLastError();

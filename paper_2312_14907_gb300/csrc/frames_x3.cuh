@@ -1,4 +1,5 @@
-// frames_x3.cuh -- the fused frame kernel for M = 128 (A2-A7 of frames.cuh)
+// frames_x3.cuh -- the fused frame kernel for M = 128 (A2-A7 of frames.cuh,
+// and the forward model A2-A3)
 // with each 2-D transform computed in three register layouts joined by two
 // shared-memory exchanges, in place of the radix-2 stages across threads
 // (warp shuffles and selects) of frames_t4.cuh.
@@ -72,6 +73,8 @@ struct X3Cfg {
   static constexpr int BUF = (B_VALS > PATCH_VALS ? B_VALS : PATCH_VALS) * (int)sizeof(cf);
   static constexpr int ABUF = M * M * (int)sizeof(float);       // sqrt(y) [q1][q0]
   static constexpr int SMEM = BUF + ABUF + 128;                  // + alignment of the tile destination
+  static constexpr int LDI = M + 1;                              // forward model: row of the staged intensities
+  static constexpr int SMEM_FWD = BUF + M * LDI * (int)sizeof(float) + 128;
   static constexpr uint32_t TMEM_COLS = 512;                     // probe (0..255), gradient window (256..)
   static constexpr uint32_t ACC_COL = 256;
   static_assert(A_VALS <= B_VALS && BUF % 16 == 0, "layouts");
@@ -236,10 +239,11 @@ MPBP_DI void x3_fetch_patch_tma(const X3Roles& r, const FrameRef& fr, cf* buf, c
   }
 }
 
-// inputs of frame fr: the patch tile and sqrt(y) [q1][q0] (64 KB); TMA: one
-// thread issues a tile load and one bulk copy on the block's mbarrier, after
-// the barrier that freed the buffers; else cp.async by every thread
-template <bool TMA>
+// inputs of frame fr: the patch tile and, but for the forward model, sqrt(y)
+// [q1][q0] (64 KB); TMA: one thread issues a tile load and one bulk copy on
+// the block's mbarrier, after the barrier that freed the buffers; else
+// cp.async by every thread
+template <bool TMA, bool FWD = false>
 MPBP_DI void x3_fetch(const FrameArgs& p, const X3Roles& r, const FrameRef& fr, cf* buf, float* abuf,
                       const BulkState& bs, const TmaMap* tm) {
   using C = X3Cfg;
@@ -247,12 +251,12 @@ MPBP_DI void x3_fetch(const FrameArgs& p, const X3Roles& r, const FrameRef& fr, 
   if constexpr (TMA) {
     if (r.tid == 0) {
       constexpr uint32_t kPatch = M * C::PW * (uint32_t)sizeof(cf);
-      constexpr uint32_t kAmp = M * M * (uint32_t)sizeof(float);
+      constexpr uint32_t kAmp = FWD ? 0u : M * M * (uint32_t)sizeof(float);
       fence_async_smem();
       mbar_arrive_tx(bs.bar, (fr.valid ? kPatch + kAmp : 0u) + tm->tx_extra);
       if (fr.valid) {
         tile_load_3d(smem_addr(buf), &tm->map, fr.s.y - (fr.s.y & 1), fr.s.x, fr.mpk, bs.bar);
-        bulk_load_stream(smem_addr(abuf), p.aT + (long long)fr.f * M * M, kAmp, bs.bar);
+        if constexpr (!FWD) bulk_load_stream(smem_addr(abuf), p.aT + (long long)fr.f * M * M, kAmp, bs.bar);
       }
     }
   } else {
@@ -262,7 +266,7 @@ MPBP_DI void x3_fetch(const FrameArgs& p, const X3Roles& r, const FrameRef& fr, 
       const int k0 = 4 * n + r.h;
       fetch_patch_elem(q, k0, r.c, buf + k0 * C::PW + r.c);
     }
-    if (q.amp) {
+    if (!FWD && q.amp) {
 #pragma unroll
       for (int i = 0; i < M * M / 4 / C::T; ++i) {
         const int ch = r.tid + i * C::T;
@@ -272,10 +276,10 @@ MPBP_DI void x3_fetch(const FrameArgs& p, const X3Roles& r, const FrameRef& fr, 
   }
 }
 
-// One frame's loss and gradient (inputs in flight); fetches the next frame's
-// inputs as soon as their buffers are free.  TMA: a wait that runs out clears
-// bs.ok and returns at once.
-template <bool TMA, bool LOSS, bool BG, bool DET, typename AddLoss>
+// One frame's loss and gradient (inputs in flight; FWD: its intensities to
+// p.I_out instead); fetches the next frame's inputs as soon as their buffers
+// are free.  TMA: a wait that runs out clears bs.ok and returns.
+template <bool TMA, bool LOSS, bool BG, bool DET, bool FWD, typename AddLoss>
 MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur, const FrameRef& nxt,
                       AddLoss&& add_loss, BulkState& bs, const TmaMap* tm, cf* buf, float* abuf, uint32_t tp,
                       uint32_t ta, const X3Tables& tab, X3Win& win) {
@@ -328,7 +332,7 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
       buf[x3_a(r.h, kp, r.c)] = v[ct::brev<32>(kp)];   // Y(h, k', c)
     });
   });
-  if constexpr (!LOSS) {
+  if constexpr (!LOSS && !FWD) {
     // the window moves to this frame's rows: rows that leave it go out
     // (here, where few registers are live, beside other warps' stores)
     if (cur.valid) {
@@ -362,7 +366,7 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
   } else {
     __syncthreads();
   }
-  if constexpr (!LOSS) tmem_fence_after_sync();
+  if constexpr (!LOSS && !FWD) tmem_fence_after_sync();
 
   // ---- L2: twiddle, 4-point over h, 8-point over c_a, twiddle
   sfor<0, 8>([&](auto a_) {
@@ -408,10 +412,40 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
     constexpr int i = decltype(i_)::value;
     v[i] = buf[x3_b(r.mt + 4 * (i / 16), r.q0, i % 16)];
   });
-  float fl = 0.0f;
   // BG: the background b of Eq. 2 (a kernel of its own, so that the common
   // case carries no per-value test)
   const float* bg = BG ? p.bgT + (long long)cur.f * M * M : nullptr;
+  if constexpr (FWD) {
+    __syncthreads();   // every layout-B read is done, and the last frame's reads of the staging
+    x3_fetch<TMA, true>(p, r, nxt, buf, abuf, bs, tm);
+    if constexpr (!TMA) cp_async_commit();
+    // I = |Psi|^2 + b through shared rows of M + 1, so that 32 consecutive q0
+    // are written, and 32 consecutive q1 read, in distinct banks; the frame
+    // then leaves in rows of 512 bytes
+    sfor<0, 2>([&](auto m_) {
+      constexpr int mr = decltype(m_)::value;
+      cf t16[16];
+      sfor<0, 16>([&](auto i_) { t16[decltype(i_)::value] = v[mr * 16 + decltype(i_)::value]; });
+      fft_line<16>(t16);
+      sfor<0, 16>([&](auto i_) {
+        constexpr int mm = decltype(i_)::value;
+        const int q1 = r.mt + 4 * mr + 8 * mm;
+        const cf z = t16[ct::brev<16>(mm)];
+        float I = fmaf(z.x, z.x, z.y * z.y);
+        if constexpr (BG) I += bg[q1 * M + r.q0];
+        abuf[r.q0 * C::LDI + q1] = I;
+      });
+    });
+    __syncthreads();
+    if (cur.valid) {
+      float* out = p.I_out + (long long)cur.f * M * M + r.tid;
+      const float* in = abuf + (r.tid >> 7) * C::LDI + (r.tid & 127);
+#pragma unroll
+      for (int i = 0; i < M * M / C::T; ++i) __stcs(out + i * C::T, in[i * (C::T / M) * C::LDI]);
+    }
+    return;
+  }
+  float fl = 0.0f;
   sfor<0, 2>([&](auto m_) {
     constexpr int mr = decltype(m_)::value;
     cf t16[16], z16[16];
@@ -536,7 +570,8 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
   tmem_fence_before_sync();
 }
 
-// loss and gradient (LOSS: loss only; BG: with the background of Eq. 2;
+// loss and gradient (LOSS: loss only; FWD: the forward model; BG: with the
+// background of Eq. 2;
 // DET: the gradient through the deterministic plan p.det): a
 // persistent grid, block b taking frames [N b / G, N (b + 1) / G) of the
 // order given (p.frames, else 0..N-1); TMA: inputs by tile and bulk copies
@@ -544,7 +579,7 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
 // thread sit in tensor memory and are reloaded when the frame's probe
 // changes: once per block for one probe, per peak for one probe per peak,
 // per frame for probes shifted per scan position.
-template <bool TMA, bool LOSS = false, bool BG = false, bool DET = false>
+template <bool TMA, bool LOSS = false, bool BG = false, bool DET = false, bool FWD = false>
 __global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, const __grid_constant__ TmaMap tm) {
   using C = X3Cfg;
   constexpr int M = C::M;
@@ -571,7 +606,7 @@ __global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, cons
   // is columns 256 + 2 s, + 1 (every warp holding column c reaches them)
   const uint32_t tp = tmem_addr(tmem_base, 32u * (warp & 3), 64u * (warp >> 2));
   const uint32_t ta = tmem_addr(tmem_base, 32u * (warp & 3), C::ACC_COL);
-  if constexpr (!LOSS) {
+  if constexpr (!LOSS && !FWD) {
     // clear the window: warp w the slots 32 (w / 4) .. + 31 of its lanes
     const uint32_t z[16] = {};
     sfor<0, 4>([&](auto k_) { tmem_st16(ta + 64u * (warp >> 2) + 16u * decltype(k_)::value, z); });
@@ -585,7 +620,7 @@ __global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, cons
   const int hi = (int)((long long)p.nframes * (blockIdx.x + 1) / gridDim.x);
   const FrameRef none = frame_ref(p, p.nframes);   // not valid: nothing to fetch
   FrameRef cur = lo < hi ? frame_ref(p, lo) : none;
-  x3_fetch<TMA>(p, r, cur, buf, abuf, bs, &tm);
+  x3_fetch<TMA, FWD>(p, r, cur, buf, abuf, bs, &tm);
   if constexpr (!TMA) cp_async_commit();
   // frame indices are read one frame ahead of their scan positions, so that
   // neither global load waits on the other
@@ -601,7 +636,7 @@ __global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, cons
         tp_src = P;
       }
     }
-    x3_frame<TMA, LOSS, BG, DET>(p, r, cur, nxt, [&](float fl) { lsum += (double)fl; }, bs, &tm, buf, abuf, tp, ta,
+    x3_frame<TMA, LOSS, BG, DET, FWD>(p, r, cur, nxt, [&](float fl) { lsum += (double)fl; }, bs, &tm, buf, abuf, tp, ta,
                             tab, win);
     if (TMA && !bs.ok) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrTimeout);
@@ -610,15 +645,17 @@ __global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, cons
     cur = nxt;
   }
   cp_async_wait_all();
-  if constexpr (!LOSS) {
+  if constexpr (!LOSS && !FWD) {
     if (bs.ok && win.ok) {   // what is left of the window
       __syncthreads();
       tmem_fence_after_sync();
       x3_flush<DET>(p, r, win, win.x, M, ta, false);
     }
   }
-  const double tot = block_sum_d<C::T>(lsum, red);
-  if (threadIdx.x == 0) p.loss_part[blockIdx.x] = tot;
+  if constexpr (!FWD) {
+    const double tot = block_sum_d<C::T>(lsum, red);
+    if (threadIdx.x == 0) p.loss_part[blockIdx.x] = tot;
+  }
   tmem_fence_before_sync();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem_base, C::TMEM_COLS);
