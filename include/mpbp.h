@@ -105,9 +105,11 @@ typedef struct {
   int32_t launches_step;      /* kernels + memsets enqueued by mpbp_step       */
   int32_t precision;          /* MPBP_PRECISION_* of the gradient evaluations */
   int32_t tile_copies;        /* FFT kernels that take their inputs by TMA tile and
-                                 bulk copies: bit 0 the gradient kernel, bit 1 the
-                                 forward kernel (none when a row of O is not a
-                                 multiple of 16 bytes, i.e. odd n2: cp.async)  */
+                                 bulk copies of unpadded rows: bit 0 the gradient
+                                 kernel, bit 1 the forward kernel (none when a row
+                                 of n2 values is not a multiple of 16 bytes, i.e.
+                                 odd n2: the context then keeps O in rows of
+                                 n2 + 1, and the tile copies read those)       */
   int32_t fft_schedule;       /* MPBP_FFT_* in use (frame side 128)            */
   int32_t deterministic;      /* 1: the gradient sums are bitwise reproducible
                                  (mpbp_set_deterministic)                     */
@@ -432,8 +434,8 @@ mpbp_status mpbp_set_fft_schedule(mpbp_ctx *ctx, int32_t schedule);
  * on a 1024^2 object; 8 x 64 x (rows + 64) at side 64),
  * allocated here and kept while the context lives, and the clearing and
  * summing of it on each evaluation.  Needs frame side 64 or 128 on FP32 FFTs
- * (at 128 the exchange schedule) and tile copies (rows of O a multiple of 16
- * bytes): else MPBP_ERR_UNSUPPORTED.  While on, evaluations over a frame list
+ * (at 128 the exchange schedule) and rows of n2 values that are a multiple of
+ * 16 bytes (even n2): else MPBP_ERR_UNSUPPORTED.  While on, evaluations over a frame list
  * (mpbp_loss_grad with frames, mpbp_adam_step minibatches), the host-buffer
  * calls, mpbp_loss_grad_batched and mpbp_autotune return
  * MPBP_ERR_UNSUPPORTED, and so do mpbp_set_precision / mpbp_set_fft_schedule
@@ -480,7 +482,7 @@ mpbp_status mpbp_set_precision(mpbp_ctx *ctx, int32_t mode);
  * never arrives at a grid barrier (the others' 0.1 s waits run out).  The
  * next mpbp_sync_status returns MPBP_ERR_TIMEOUT.  Results of calls made
  * while it is on are meaningless.  No effect on contexts whose frame kernels
- * use cp.async copies (odd n2, M <= 16).  Off by default. */
+ * use cp.async copies (M <= 16).  Off by default. */
 mpbp_status mpbp_set_test_stall(mpbp_ctx *ctx, int32_t on);
 
 /* Turns on (enable != 0) or off the recording of CUDA events around every

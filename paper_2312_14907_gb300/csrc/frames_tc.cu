@@ -221,14 +221,14 @@ struct TcGroup {
 
 // next frame's object patch and sqrt(y) tile into the staging buffers
 MPBP_DI void fetch_patch(const FrameArgs& p, const TcGroup& G, const FrameRef& r) {
-  const cf* obj = p.O + r.mpk * p.obj_stride;
+  const cf* obj = p.O + r.mpk * p.o_stride;
 #pragma unroll 4
   for (int i = 0; i < TM * TM / GT; ++i) {
     const int e = G.t + i * GT;
     const int k0 = e >> 6, k1 = e & 63;
     const int row = r.s.x + k0, col = r.s.y + k1;
     const bool ok = r.valid && row >= 0 && row < p.n1 && col >= 0 && col < p.n2;
-    cp_async8(G.patch + patch_idx(k0, k1), ok ? obj + (long long)row * p.n2 + col : obj, ok);
+    cp_async8(G.patch + patch_idx(k0, k1), ok ? obj + (long long)row * p.o_pitch + col : obj, ok);
   }
   cp_async_commit();
 }
@@ -258,10 +258,10 @@ MPBP_DI void fetch_patch4(const FrameArgs& p, const TcGroup& G, const FrameRef (
     const int e = G.t + i * GT;
     const int k0 = e >> 6, k1 = e & 63;
     const FrameRef& fr = r[2 * (k0 >> 5) + (k1 >> 5)];
-    const cf* obj = p.O + fr.mpk * p.obj_stride;
+    const cf* obj = p.O + fr.mpk * p.o_stride;
     const int row = fr.s.x + (k0 & 31), col = fr.s.y + (k1 & 31);
     const bool ok = fr.valid && row >= 0 && row < p.n1 && col >= 0 && col < p.n2;
-    cp_async8(G.patch + patch_idx(k0, k1), ok ? obj + (long long)row * p.n2 + col : obj, ok);
+    cp_async8(G.patch + patch_idx(k0, k1), ok ? obj + (long long)row * p.o_pitch + col : obj, ok);
   }
   cp_async_commit();
 }
@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   for (int it = NGROUPS * blockIdx.x + gi; it < p.nframes && G.ok; it += stride) {
     const FrameRef cur = frame_ref(p, it);
     const cf* P = frame_probe(p, cur, FS * FS);
-    const cf* obj = p.O + cur.mpk * p.obj_stride;
+    const cf* obj = p.O + cur.mpk * p.o_stride;
     for (int ab = 0; ab < 4 && G.ok; ++ab) {
       const int a = ab >> 1, b = ab & 1;
       group_bar(G.id);   // the staging tile's last reads (previous residual) are done
@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             const int row = cur.s.x + r0, col = cur.s.y + c0;
             cf psi = cf{0.0f, 0.0f};
             if (cur.valid && row >= 0 && row < p.n1 && col >= 0 && col < p.n2)
-              psi = cmul(ldg_cf(P + r0 * FS + c0), ldg_cf(obj + (long long)row * p.n2 + col));
+              psi = cmul(ldg_cf(P + r0 * FS + c0), ldg_cf(obj + (long long)row * p.o_pitch + col));
             if ((a * i + b * jj) & 1) sum = csub(sum, psi);
             else sum = cadd(sum, psi);
           }

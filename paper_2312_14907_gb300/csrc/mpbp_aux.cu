@@ -18,7 +18,10 @@ namespace mpbp {
 template <bool PHI>
 __global__ void object_build_kernel(ObjectArgs a) {
   const long long stride = (long long)gridDim.x * blockDim.x;
+  const int pad = a.pitch - a.n2;
+  const long long ostride = a.npix / a.n2 * a.pitch;
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < a.npix; p += stride) {
+    const long long q = pad ? p + (unsigned)p / (unsigned)a.n2 * (long long)pad : p;   // npix < 2^31
     const float r = a.rho[p];
     float uc[kMaxComp];
 #pragma unroll
@@ -36,7 +39,7 @@ __global__ void object_build_kernel(ObjectArgs a) {
           sincospif(arg, &sn, &cs);   // exp(i phi), phi = pi * arg
         }
         const float amp = a.alpha[m] * r;
-        reinterpret_cast<float2*>(a.O)[m * a.npix + p] = make_float2(amp * cs, amp * sn);
+        reinterpret_cast<float2*>(a.O)[m * ostride + q] = make_float2(amp * cs, amp * sn);
       }
     }
   }

@@ -41,7 +41,7 @@ inline mpbp_status validate_problem(const mpbp_problem* pr) {
 
 // Arguments of the fused per-frame kernel (A2..A7 of the hot path).
 struct FrameArgs {
-  const cf* O;          // [D][n1][n2] objects O_m
+  const cf* O;          // [D][n1][o_pitch] objects O_m
   const cf* probe;      // [Dp][M][M]
   const float* aT;      // [D*J][M][M] sqrt(y), each frame stored transposed [q1][q0]
   const float* bgT;     // same layout as aT, or nullptr
@@ -54,10 +54,12 @@ struct FrameArgs {
   unsigned* arrivals;   // block counter of the gradient assembly that follows;
                         // cleared here, before that kernel can start
   long long obj_stride; // n1*n2
+  long long o_stride;   // n1*o_pitch
   int nframes;          // frames to process
   int frame0;           // without a frame list: frames frame0 .. frame0 + nframes - 1
   int nframes_total;    // D*J (bound for frame indices)
   int n1, n2, J;
+  int o_pitch;          // row of O: n2, or n2 + 1 where that makes 16-byte rows
   int probe_stride;     // M*M when one probe per peak, 0 when one for all;
                         // kProbePerScan / kProbePerFrame: one per scan
                         // position j / per frame f, M*M apart (scan
@@ -108,8 +110,9 @@ struct ObjectArgs {
   const float* u;
   const float* phi;     // per-peak phases [D][npix] in place of u (or nullptr)
   const float* alpha;
-  cf* O;
+  cf* O;                // [D][npix / n2][pitch]
   long long npix;
+  int n2, pitch;
   int D, C;
   PhaseCoef pc;
 };

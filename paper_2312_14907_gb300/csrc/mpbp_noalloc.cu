@@ -129,6 +129,7 @@ extern "C" mpbp_status mpbp_loss_grad_noalloc(const mpbp_problem* pr, const floa
   oa.u = u;
   oa.alpha = alpha;
   oa.O = O;
+  oa.n2 = oa.pitch = pr->n2;
   oa.npix = npix;
   oa.D = pr->npeaks;
   oa.C = pr->ncomp;
@@ -148,6 +149,8 @@ extern "C" mpbp_status mpbp_loss_grad_noalloc(const mpbp_problem* pr, const floa
   fa.err = err;
   fa.arrivals = arrivals;
   fa.obj_stride = npix;
+  fa.o_stride = npix;
+  fa.o_pitch = pr->n2;
   fa.nframes = (int)nframes;
   fa.frame0 = 0;
   fa.nframes_total = (int)nframes;
