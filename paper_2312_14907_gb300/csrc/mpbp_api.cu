@@ -122,11 +122,10 @@ struct mpbp_ctx {
   bool shift_ready = false;
   // optional event timing of the fused frame kernel
   bool timing = false;
-  // Alg. 1: Adam moments and the materialised rho, alpha (mpbp_adam_init)
+  // Alg. 1: Adam moments (mpbp_adam_init)
   void* adam_buf = nullptr;
   float *m_chi = nullptr, *v_chi = nullptr, *m_u = nullptr, *v_u = nullptr;
   double *m_a = nullptr, *v_a = nullptr;
-  float *rho_x = nullptr, *alpha_x = nullptr;
   // phase unwrapping / projector workspace (lazily allocated)
   void* uw_buf = nullptr;
   UnwrapArgs uw{};
@@ -481,7 +480,7 @@ mpbp_status enqueue_probe_shift(mpbp_ctx* c, cudaStream_t s) {
 
 mpbp_status enqueue_object_build(mpbp_ctx* c, const float* rho, const float* u,
                                  const float* alpha, cf* out, cudaStream_t s,
-                                 const float* phi = nullptr) {
+                                 const float* phi = nullptr, const AdamArgs* adam = nullptr) {
   ObjectArgs oa{};
   oa.rho = rho;
   oa.u = u;
@@ -494,25 +493,28 @@ mpbp_status enqueue_object_build(mpbp_ctx* c, const float* rho, const float* u,
   oa.D = c->D;
   oa.C = c->C;
   oa.pc = c->pc;
+  if (adam) oa.ad = *adam;
   MPBP_CUDA(c, launch_object_build(oa, c->num_sms, s));
   return MPBP_OK;
 }
 
 // A1..A8: objects, fused frames, gradient assembly, reductions.  st != nullptr
-// adds the line-search decision, and step (with st) the optimizer update.
+// adds the line-search decision, and step (with st) the optimizer update;
+// adam takes rho and alpha from the Adam variables and updates them in place
+// of writing gradients.
 mpbp_status enqueue_loss_grad(mpbp_ctx* c, const float* rho, const float* u, const float* alpha,
                               const int32_t* frames, int32_t nframes, double* loss,
                               float* g_rho, float* g_u, double* g_alpha,
                               mpbp_step_state* st, cudaStream_t s,
                               const float* phi = nullptr, float* g_phi = nullptr,
-                              const StepPtrs* step = nullptr) {
+                              const StepPtrs* step = nullptr, const AdamArgs* adam = nullptr) {
   if (c->det && frames)
     return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient is for evaluations over every frame");
   if (c->acc_dirty) {
     MPBP_CUDA(c, cudaMemsetAsync(c->acc, 0, sizeof(cf) * c->npix * c->D, s));
     c->acc_dirty = false;
   }
-  mpbp_status r = enqueue_object_build(c, rho, u, alpha, c->O, s, phi);
+  mpbp_status r = enqueue_object_build(c, rho, u, alpha, c->O, s, phi, adam);
   if (r != MPBP_OK) return r;
   const int nf = frames ? nframes : (int)c->nframes;
   FrameArgs fa = frame_args(c, frames, nf);
@@ -562,6 +564,7 @@ mpbp_status enqueue_loss_grad(mpbp_ctx* c, const float* rho, const float* u, con
   ra.st = st;
   ra.alpha_from = 1;
   if (step) ra.step = *step;
+  if (adam) fi.ad = ra.ad = *adam;
   MPBP_CUDA(c, launch_finish(fi, ra, c->finish_grid, s));
   c->acc_dirty = false;
   return MPBP_OK;
@@ -1317,8 +1320,7 @@ mpbp_status mpbp_adam_init(mpbp_ctx* c, const mpbp_adam_params* prm, mpbp_adam_s
   if (!c->adam_buf) {
     Carver cv;
     const size_t o_mc = cv.take<float>(np), o_vc = cv.take<float>(np), o_mu = cv.take<float>(nu),
-                 o_vu = cv.take<float>(nu), o_ma = cv.take<double>(c->D), o_va = cv.take<double>(c->D),
-                 o_rx = cv.take<float>(np), o_ax = cv.take<float>(c->D);
+                 o_vu = cv.take<float>(nu), o_ma = cv.take<double>(c->D), o_va = cv.take<double>(c->D);
     void* b = nullptr;
     MPBP_CUDA(c, cudaStreamSynchronize(s));
     if (cudaMalloc(&b, align_up(cv.off, 256)) != cudaSuccess) {
@@ -1333,8 +1335,6 @@ mpbp_status mpbp_adam_init(mpbp_ctx* c, const mpbp_adam_params* prm, mpbp_adam_s
     c->v_u = reinterpret_cast<float*>(p + o_vu);
     c->m_a = reinterpret_cast<double*>(p + o_ma);
     c->v_a = reinterpret_cast<double*>(p + o_va);
-    c->rho_x = reinterpret_cast<float*>(p + o_rx);
-    c->alpha_x = reinterpret_cast<float*>(p + o_ax);
   }
   MPBP_CUDA(c, cudaMemsetAsync(c->m_chi, 0, sizeof(float) * np, s));
   MPBP_CUDA(c, cudaMemsetAsync(c->v_chi, 0, sizeof(float) * np, s));
@@ -1367,11 +1367,6 @@ mpbp_status mpbp_adam_step(mpbp_ctx* c, const int32_t* frames, int32_t nframes, 
   a.u = u;
   a.alpha_t = alpha_t;
   a.mask = mask;
-  a.rho_x = c->rho_x;
-  a.alpha_x = c->alpha_x;
-  a.g_rho = c->g_rho_ws;
-  a.g_u = c->g_u_ws;
-  a.g_alpha = c->g_alpha_ws;
   a.m_chi = c->m_chi;
   a.v_chi = c->v_chi;
   a.m_u = c->m_u;
@@ -1379,15 +1374,8 @@ mpbp_status mpbp_adam_step(mpbp_ctx* c, const int32_t* frames, int32_t nframes, 
   a.m_a = c->m_a;
   a.v_a = c->v_a;
   a.st = st;
-  a.npix = c->npix;
-  a.C = c->C;
-  a.D = c->D;
-  MPBP_CUDA(c, launch_adam_prep(a, c->num_sms, s));
-  mpbp_status r = enqueue_loss_grad(c, c->rho_x, u, c->alpha_x, frames, frames ? nframes : 0, &st->f_last,
-                                    c->g_rho_ws, c->g_u_ws, nullptr, nullptr, s);
-  if (r != MPBP_OK) return r;
-  MPBP_CUDA(c, launch_adam_update(a, c->num_sms, s));
-  return MPBP_OK;
+  return enqueue_loss_grad(c, nullptr, u, nullptr, frames, frames ? nframes : 0, &st->f_last, nullptr, nullptr,
+                           nullptr, nullptr, s, nullptr, nullptr, nullptr, &a);
 }
 
 mpbp_status mpbp_adam_get_state(mpbp_ctx* c, float* m_chi, float* v_chi, float* m_u, float* v_u,

@@ -13,24 +13,75 @@ namespace mpbp {
 // ----------------------------------------------------------------------------
 // A1: objects
 // ----------------------------------------------------------------------------
-// PHI: the phases phi_m are given per peak (the per-peak-phase variables of
-// the paper's two-step reconstruction) instead of derived from u
-template <bool PHI>
+// 1 - b^t for 0 <= b < 1, t >= 1: binary powers, each kept as an FP64 pair
+// (hi + lo), so that the result is good to an ulp or two for every t; the
+// loop is far shorter than the library's pow, whose latency one thread would
+// put in front of the whole step (minibatch step 47 -> 26 us with the
+// fusions below, see the Adam form of the object synthesis).
+__device__ double one_minus_pow(double b, long long t) {
+  struct Dd {
+    double h, l;
+  };
+  auto mul = [](Dd x, Dd y) {
+    const double p = x.h * y.h;
+    const double e = fma(x.h, y.h, -p) + fma(x.h, y.l, x.l * y.h);
+    const double h = p + e;
+    return Dd{h, e - (h - p)};
+  };
+  Dd r{1.0, 0.0}, x{b, 0.0};
+  while (true) {
+    if (t & 1) r = mul(r, x);
+    t >>= 1;
+    if (t == 0) break;
+    x = mul(x, x);
+  }
+  return (1.0 - r.h) - r.l;
+}
+
+// Where the phases and amplitudes of O come from.
+enum ObjectForm {
+  kObjU,     // rho, alpha; phases from u
+  kObjPhi,   // rho, alpha; phases phi_m per peak (the per-peak-phase variables
+             // of the paper's two-step reconstruction)
+  kObjAdam   // rho = mask e^chi, alpha = (1, e^alpha_t) of Eq. 8, phases from u;
+             // block 0 also counts the Adam step
+};
+
+template <int FORM>
 __global__ void object_build_kernel(ObjectArgs a) {
   const long long stride = (long long)gridDim.x * blockDim.x;
   const int pad = a.pitch - a.n2;
   const long long ostride = a.npix / a.n2 * a.pitch;
+  __shared__ float s_alpha[kMaxPeaks];
+  if (threadIdx.x < a.D) {
+    const int m = threadIdx.x;
+    if constexpr (FORM == kObjAdam) s_alpha[m] = m == 0 ? 1.0f : expf(a.ad.alpha_t[m]);
+    else s_alpha[m] = a.alpha[m];
+  }
+  if (FORM == kObjAdam && blockIdx.x == 0) {
+    mpbp_adam_state* st = a.ad.st;
+    const long long t = st->t + 1;
+    __syncthreads();   // every thread has read the old count
+    if (threadIdx.x == 0) {
+      st->t = t;
+      st->bc1 = one_minus_pow(st->beta1, t);
+    }
+    if (threadIdx.x == 32) st->bc2 = one_minus_pow(st->beta2, t);
+  }
+  __syncthreads();
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < a.npix; p += stride) {
     const long long q = pad ? p + (unsigned)p / (unsigned)a.n2 * (long long)pad : p;   // npix < 2^31
-    const float r = a.rho[p];
+    float r;
+    if constexpr (FORM == kObjAdam) r = (a.ad.mask ? a.ad.mask[p] : 1.0f) * expf(a.ad.chi[p]);
+    else r = a.rho[p];
     float uc[kMaxComp];
 #pragma unroll
-    for (int c = 0; c < kMaxComp; ++c) uc[c] = !PHI && c < a.C ? a.u[c * a.npix + p] : 0.f;
+    for (int c = 0; c < kMaxComp; ++c) uc[c] = FORM != kObjPhi && c < a.C ? a.u[c * a.npix + p] : 0.f;
 #pragma unroll
     for (int m = 0; m < kMaxPeaks; ++m) {
       if (m < a.D) {
         float sn, cs;
-        if constexpr (PHI) {
+        if constexpr (FORM == kObjPhi) {
           sincosf(a.phi[m * a.npix + p], &sn, &cs);
         } else {
           float arg = 0.f;
@@ -38,7 +89,7 @@ __global__ void object_build_kernel(ObjectArgs a) {
           for (int c = 0; c < kMaxComp; ++c) arg = fmaf(a.pc.kpi[m][c], uc[c], arg);
           sincospif(arg, &sn, &cs);   // exp(i phi), phi = pi * arg
         }
-        const float amp = a.alpha[m] * r;
+        const float amp = s_alpha[m] * r;
         reinterpret_cast<float2*>(a.O)[m * ostride + q] = make_float2(amp * cs, amp * sn);
       }
     }
@@ -160,12 +211,27 @@ __device__ StepDecision step_decide(const StepView& st, double loss) {
   return d;
 }
 
+// What the gradient assembly writes.
+enum FinishForm {
+  kFinGrad,   // df/drho, df/du
+  kFinPhi,    // df/drho, df/dphi_m
+  kFinStep,   // also mpbp_step's update x = x_base - t w g_base, after a decision
+              // that every block takes from the same fixed-order loss sum (the
+              // last block updates alpha and records the state)
+  kFinAdam    // mpbp_adam_step's update in place of the gradients: the chain rule to
+              // the auxiliary variables, g_chi = rho df/drho, g_alpha_t[m] =
+              // alpha_m df/dalpha_m, then Adam (Kingma and Ba) on chi, u and
+              // alpha_t[1..D-1], moments in FP32 per pixel and FP64 per peak,
+              // bias corrections in FP64
+};
+
 // STEP: the loss is the block's own fixed-order sum of all frame-kernel
 // partials (loss_all), and the alpha update of the step follows the decision
 // (thread m updates alpha_m).  The state and the alpha values are read
 // before the partials, so their latency overlaps the partial sums.
-template <int T, bool STEP>
+template <int T, int FORM>
 __device__ void final_reduce(const ReduceArgs& a, double loss_all) {
+  constexpr bool STEP = FORM == kFinStep;
   __shared__ double vals[kMaxPeaks + 3];
   __shared__ int s_accept;
   __shared__ double s_step;   // t_new * w_alpha
@@ -241,45 +307,90 @@ __device__ void final_reduce(const ReduceArgs& a, double loss_all) {
       x.alpha[m] = m < a.alpha_from ? (float)base : (float)(base - s_step * gbase);
     }
   }
+  if constexpr (FORM == kFinAdam) {
+    // alpha_t[0] is not a variable (alpha_0 = 1): its gradient is 0 and it
+    // never moves, so it is left alone
+    const int m = threadIdx.x;
+    if (m >= 1 && m < a.D) {
+      const AdamArgs& d = a.ad;
+      const mpbp_adam_state* as = d.st;
+      const float at = d.alpha_t[m];
+      const double g = (double)expf(at) * galpha[m];
+      const double mo = as->beta1 * d.m_a[m] + (1.0 - as->beta1) * g;
+      const double ve = as->beta2 * d.v_a[m] + (1.0 - as->beta2) * g * g;
+      d.m_a[m] = mo;
+      d.v_a[m] = ve;
+      d.alpha_t[m] = (float)((double)at - as->lr_alpha * (mo / as->bc1) / (sqrt(ve / as->bc2) + as->eps));
+    }
+  }
 }
 
 constexpr int kFinishThreads = 256;
 constexpr int kFinishPixelsPerThread = 1;   // latency-bound: many warps, few pixels each
 
-// the loads of one pixel, issued together before its phase arithmetic
-template <bool PHI>
+// One pixel's loads, issued together before its phase arithmetic.  MP: peaks
+// held in registers (the smallest of 4, 8, 16 that holds D: with 16 the
+// kernel took 118 registers, two blocks an SM).
+template <int FORM, int MP>
 struct PixelIn {
   float r;
   float uc[kMaxComp];
-  float2 Am[kMaxPeaks];
+  float2 Am[MP];
+  float chi, mo[1 + kMaxComp], ve[1 + kMaxComp];   // Adam: log density, moments of chi and u
 };
 
-template <bool PHI>
-__device__ __forceinline__ void pixel_load(const FinishArgs& a, long long p, PixelIn<PHI>& in) {
+template <int FORM, int MP>
+__device__ __forceinline__ void pixel_load(const FinishArgs& a, long long p, PixelIn<FORM, MP>& in) {
   const float2* acc = reinterpret_cast<const float2*>(a.acc);
-  in.r = a.rho[p];
+  if constexpr (FORM == kFinAdam) {
+    in.r = a.ad.mask ? a.ad.mask[p] : 1.0f;
+    in.chi = a.ad.chi[p];
+    in.mo[0] = a.ad.m_chi[p];
+    in.ve[0] = a.ad.v_chi[p];
 #pragma unroll
-  for (int c = 0; c < kMaxComp; ++c) in.uc[c] = !PHI && c < a.C ? a.u[c * a.npix + p] : 0.f;
+    for (int c = 0; c < kMaxComp; ++c) {
+      if (c < a.C) {
+        in.mo[1 + c] = a.ad.m_u[c * a.npix + p];
+        in.ve[1 + c] = a.ad.v_u[c * a.npix + p];
+      }
+    }
+  } else {
+    in.r = a.rho[p];
+  }
 #pragma unroll
-  for (int m = 0; m < kMaxPeaks; ++m) in.Am[m] = m < a.D ? __ldcg(acc + m * a.npix + p) : make_float2(0.f, 0.f);
+  for (int c = 0; c < kMaxComp; ++c) in.uc[c] = FORM != kFinPhi && c < a.C ? a.u[c * a.npix + p] : 0.f;
+#pragma unroll
+  for (int m = 0; m < MP; ++m) in.Am[m] = m < a.D ? __ldcg(acc + m * a.npix + p) : make_float2(0.f, 0.f);
 }
 
-// STEP: mpbp_step's update x = x_base - t w g_base is applied here, pixel by
-// pixel, after a decision that every block takes from the same fixed-order
-// loss sum; the last block updates alpha and records the state.
-template <bool PHI, bool STEP>
+// the Adam step of one variable with gradient g
+struct AdamCoef {
+  float b1, b2, eps, ic1, ic2, lr_chi, lr_u;
+};
+__device__ __forceinline__ void adam_var(const AdamCoef& k, float lr, float g, float x, float mo, float ve, float* xp,
+                                         float* mp, float* vp) {
+  const float m = fmaf(k.b1, mo, (1.0f - k.b1) * g);
+  const float v = fmaf(k.b2, ve, (1.0f - k.b2) * g * g);
+  *mp = m;
+  *vp = v;
+  *xp = x - lr * (m * k.ic1) / (sqrtf(v * k.ic2) + k.eps);
+}
+
+template <int FORM, int MP>
 __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, ReduceArgs ra) {
+  constexpr bool STEP = FORM == kFinStep;
   constexpr int NW = kFinishThreads / 32;
-  constexpr int NQ = kMaxPeaks + 3;
+  constexpr int NQ = MP + 3;
   __shared__ double wsum[NW][NQ];
   __shared__ double s_loss;
   __shared__ float s_w[2];
+  __shared__ float s_alpha[MP];
   __shared__ int s_accept;
   __shared__ bool last;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float ap[kMaxPeaks];   // df/dalpha_m partials of this thread
+  float ap[MP];   // df/dalpha_m partials of this thread
 #pragma unroll
-  for (int m = 0; m < kMaxPeaks; ++m) ap[m] = 0.f;
+  for (int m = 0; m < MP; ++m) ap[m] = 0.f;
   float n_rho = 0.f, n_u = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -295,8 +406,19 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
   } else {
     for (long long i = p0; i < a.n_loss_part; i += stride) lp += __ldcg(a.loss_part + i);
   }
-  PixelIn<PHI> in;
-  if (p0 < a.npix) pixel_load<PHI>(a, p0, in);
+  PixelIn<FORM, MP> in;
+  if (p0 < a.npix) pixel_load<FORM, MP>(a, p0, in);
+  if (threadIdx.x < a.D) {
+    const int m = threadIdx.x;
+    if constexpr (FORM == kFinAdam) s_alpha[m] = m == 0 ? 1.0f : expf(a.ad.alpha_t[m]);
+    else s_alpha[m] = a.alpha[m];
+  }
+  AdamCoef ak{};
+  if constexpr (FORM == kFinAdam) {
+    const mpbp_adam_state* st = a.ad.st;
+    ak = AdamCoef{(float)st->beta1,       (float)st->beta2,  (float)st->eps, (float)(1.0 / st->bc1),
+                  (float)(1.0 / st->bc2), (float)st->lr_chi, (float)st->lr_u};
+  }
   if (!STEP || w == 0) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) lp += __shfl_xor_sync(0xffffffffu, lp, o);
@@ -311,21 +433,23 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
       s_w[0] = (float)(d.t_new * sv.w_rho);
       s_w[1] = (float)(d.t_new * sv.w_u);
     }
-    __syncthreads();
+  }
+  __syncthreads();
+  if constexpr (STEP) {
     accept = s_accept != 0;
     wr = s_w[0];
     wu = s_w[1];
   }
   float2* acc = reinterpret_cast<float2*>(a.acc);
   for (long long p = p0; p < a.npix; p += stride) {
-    const float r = in.r;
+    const float r = FORM == kFinAdam ? in.r * expf(in.chi) : in.r;
     float gr = 0.f, gphi2 = 0.f;
     float gu[kMaxComp] = {0.f, 0.f, 0.f};
 #pragma unroll
-    for (int m = 0; m < kMaxPeaks; ++m) {
+    for (int m = 0; m < MP; ++m) {
       if (m < a.D) {
         float sn, cs;
-        if constexpr (PHI) {
+        if constexpr (FORM == kFinPhi) {
           sincosf(a.phi[m * a.npix + p], &sn, &cs);
         } else {
           float arg = 0.f;
@@ -337,10 +461,10 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
         acc[m * a.npix + p] = make_float2(0.f, 0.f);
         const float Tr = fmaf(cs, A.x, -sn * A.y);
         const float Ti = fmaf(cs, A.y, sn * A.x);
-        const float am = a.alpha[m];
+        const float am = s_alpha[m];
         gr = fmaf(am, Tr, gr);
         const float dphi = -am * r * Ti;
-        if constexpr (PHI) {
+        if constexpr (FORM == kFinPhi) {
           a.g_phi[m * a.npix + p] = dphi;
           gphi2 = fmaf(dphi, dphi, gphi2);
         } else {
@@ -350,13 +474,24 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
         ap[m] = fmaf(r, Tr, ap[m]);
       }
     }
-    a.g_rho[p] = gr;
-    float su = gphi2;   // |g_phi|^2 in the phase form, |g_u|^2 otherwise
-    if constexpr (!PHI) {
+    if constexpr (FORM == kFinAdam) {
+      adam_var(ak, ak.lr_chi, r * gr, in.chi, in.mo[0], in.ve[0], a.ad.chi + p, a.ad.m_chi + p, a.ad.v_chi + p);
 #pragma unroll
       for (int c = 0; c < kMaxComp; ++c) {
         if (c < a.C) {
-          a.g_u[c * a.npix + p] = gu[c];
+          const long long i = c * a.npix + p;
+          adam_var(ak, ak.lr_u, gu[c], in.uc[c], in.mo[1 + c], in.ve[1 + c], a.ad.u + i, a.ad.m_u + i, a.ad.v_u + i);
+        }
+      }
+    } else {
+      a.g_rho[p] = gr;
+    }
+    float su = gphi2;   // |g_phi|^2 in the phase form, |g_u|^2 otherwise
+    if constexpr (FORM != kFinPhi) {
+#pragma unroll
+      for (int c = 0; c < kMaxComp; ++c) {
+        if (c < a.C) {
+          if constexpr (FORM != kFinAdam) a.g_u[c * a.npix + p] = gu[c];
           su = fmaf(gu[c], gu[c], su);
         }
       }
@@ -393,14 +528,14 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
     }
     n_rho = fmaf(gr, gr, n_rho);
     n_u += su;
-    if (p + stride < a.npix) pixel_load<PHI>(a, p + stride, in);
+    if (p + stride < a.npix) pixel_load<FORM, MP>(a, p + stride, in);
   }
   // partial sums: FP32 within the warp (a few pixels per lane), FP64 across
   // warps and blocks; one barrier for all D + 3 quantities
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     if (q < a.D + 2) {
-      float v = q < a.D ? ap[q < kMaxPeaks ? q : 0] : (q == a.D ? n_rho : n_u);
+      float v = q < a.D ? ap[q < MP ? q : 0] : (q == a.D ? n_rho : n_u);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0) wsum[w][q] = (double)v;
@@ -421,7 +556,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
   __syncthreads();
   if (!last) return;
   __threadfence();
-  final_reduce<kFinishThreads, STEP>(ra, STEP ? s_loss : 0.0);
+  final_reduce<kFinishThreads, FORM>(ra, STEP ? s_loss : 0.0);
 }
 
 // The loss alone (mpbp_loss): one warp sums the frame kernel's per-block
@@ -599,8 +734,10 @@ static int grid_for(long long n, int threads, int cap) {
 }
 
 cudaError_t launch_object_build(const ObjectArgs& a, int num_sms, cudaStream_t s) {
-  if (a.phi) object_build_kernel<true><<<grid_for(a.npix, 256, num_sms * 8), 256, 0, s>>>(a);
-  else object_build_kernel<false><<<grid_for(a.npix, 256, num_sms * 8), 256, 0, s>>>(a);
+  const int grid = grid_for(a.npix, 256, num_sms * 8);
+  if (a.ad.chi) object_build_kernel<kObjAdam><<<grid, 256, 0, s>>>(a);
+  else if (a.phi) object_build_kernel<kObjPhi><<<grid, 256, 0, s>>>(a);
+  else object_build_kernel<kObjU><<<grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -632,17 +769,22 @@ cudaError_t launch_loss_reduce(const double* part, long long n, double* loss, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_finish(const FinishArgs& a, const ReduceArgs& r, int grid, cudaStream_t s) {
-  if (a.phi) {
-    if (r.step.rho) return cudaErrorInvalidValue;   // the step updates u, not per-peak phases
-    finish_kernel<true, false><<<grid, kFinishThreads, 0, s>>>(a, r);
-  } else if (r.step.rho) {
-    if (!r.st) return cudaErrorInvalidValue;
-    finish_kernel<false, true><<<grid, kFinishThreads, 0, s>>>(a, r);
-  } else {
-    finish_kernel<false, false><<<grid, kFinishThreads, 0, s>>>(a, r);
-  }
+template <int FORM>
+static cudaError_t launch_finish_form(const FinishArgs& a, const ReduceArgs& r, int grid, cudaStream_t s) {
+  if (a.D <= 4) finish_kernel<FORM, 4><<<grid, kFinishThreads, 0, s>>>(a, r);
+  else if (a.D <= 8) finish_kernel<FORM, 8><<<grid, kFinishThreads, 0, s>>>(a, r);
+  else finish_kernel<FORM, kMaxPeaks><<<grid, kFinishThreads, 0, s>>>(a, r);
   return cudaGetLastError();
+}
+
+cudaError_t launch_finish(const FinishArgs& a, const ReduceArgs& r, int grid, cudaStream_t s) {
+  // one form a launch: the step updates u, not per-peak phases
+  if ((a.phi && r.step.rho) || (a.ad.chi && (a.phi || r.step.rho || !a.ad.st)) || (r.step.rho && !r.st))
+    return cudaErrorInvalidValue;
+  if (a.ad.chi) return launch_finish_form<kFinAdam>(a, r, grid, s);
+  if (a.phi) return launch_finish_form<kFinPhi>(a, r, grid, s);
+  if (r.step.rho) return launch_finish_form<kFinStep>(a, r, grid, s);
+  return launch_finish_form<kFinGrad>(a, r, grid, s);
 }
 
 }  // namespace mpbp

@@ -105,6 +105,23 @@ struct PhaseCoef {
   float kps[kMaxPeaks][kMaxComp];  // phase_scale * G       (d phi_m / d u_c)
 };
 
+// Alg. 1 (Adam in the auxiliary variables of Eq. 8): with chi set, the object
+// synthesis takes rho = mask e^chi and alpha = (1, e^alpha_t[1..]) and counts
+// the step, and the gradient assembly applies the chain rule and the update
+struct AdamArgs {
+  float* chi;           // [npix] log density (updated)
+  float* u;             // [C][npix] (updated)
+  float* alpha_t;       // [D] log peak scalings, entry 0 unused (updated)
+  const float* mask;    // [npix] support, or nullptr
+  float* m_chi;         // Adam moments
+  float* v_chi;
+  float* m_u;
+  float* v_u;
+  double* m_a;
+  double* v_a;
+  mpbp_adam_state* st;  // parameters, step count, bias corrections
+};
+
 struct ObjectArgs {
   const float* rho;
   const float* u;
@@ -115,6 +132,7 @@ struct ObjectArgs {
   int n2, pitch;
   int D, C;
   PhaseCoef pc;
+  AdamArgs ad;          // ad.chi set: rho and alpha from the Adam variables
 };
 
 // Per-pixel gradient assembly (A6/A7 tail) and its partial sums.
@@ -134,6 +152,7 @@ struct FinishArgs {
   long long npix;
   int D, C;
   PhaseCoef pc;
+  AdamArgs ad;          // ad.chi set: Adam in place of the gradient outputs
 };
 
 // The optimizer update of mpbp_step, applied by the gradient assembly itself:
@@ -162,6 +181,7 @@ struct ReduceArgs {
   mpbp_step_state* st;  // nullable: decide an optimizer step
   int alpha_from;       // first alpha index that is a variable (1)
   StepPtrs step;        // with st: the iterate and base point to update
+  AdamArgs ad;          // ad.chi set: the update of alpha_t
 };
 
 }  // namespace mpbp
