@@ -501,7 +501,8 @@ mpbp_status mpbp_frames_timing_read(mpbp_ctx *ctx, double *total_ms, int32_t *co
  * side with that side's own block shape; mode 2 = as mode 1 for sides 32 and
  * 64, one launch per problem for side 128; mode 3 = one launch per problem.
  * Problems with M <= 16 always get their own launch.  order 0 = work items
- * grouped by problem, 1 = problems interleaved.  Host-side only. */
+ * grouped by problem, 1 = problems interleaved (side 128 in a launch of its
+ * own always takes each problem's column strips in turn).  Host-side only. */
 mpbp_status mpbp_set_batch_schedule(mpbp_ctx *ctx, int32_t mode, int32_t order);
 
 /* Autotuner for one context: times mpbp_loss_grad at rho, u, alpha (dev)

@@ -30,6 +30,14 @@ bool probe_shift_prepare(int m);
 cudaError_t launch_probe_shift(const ProbeShiftArgs& a, cudaStream_t s);
 
 cudaError_t launch_object_build(const ObjectArgs& a, int num_sms, cudaStream_t s);
+// several problems in one launch (objects from u; block0 is filled in)
+constexpr int kAuxBatch = 32;   // problems a launch's parameter space holds
+struct ObjectBatch {
+  ObjectArgs a[kAuxBatch];
+  int block0[kAuxBatch + 1];
+  int n;
+};
+cudaError_t launch_object_build_batch(ObjectBatch& b, int num_sms, cudaStream_t s);
 // out[i] = in[i] for n 16-bit counts
 cudaError_t launch_counts16(const unsigned short* in, float* out, long long n, int num_sms, cudaStream_t s);
 cudaError_t launch_frame_transpose(const float* in, float* out, long long nframes, int m,
@@ -39,6 +47,16 @@ int finish_grid(long long npix, int num_sms);
 // with r.step set (and r.st), also the optimizer update of mpbp_step; with
 // a.ad.chi set, the Adam update of mpbp_adam_step
 cudaError_t launch_finish(const FinishArgs& a, const ReduceArgs& r, int grid, cudaStream_t s);
+// the gradients of several problems in one launch (r[k].n_part blocks each;
+// block0 is filled in)
+struct FinishBatch {
+  FinishArgs a[kAuxBatch];
+  ReduceArgs r[kAuxBatch];
+  int block0[kAuxBatch + 1];
+  int n;
+};
+static_assert(sizeof(FinishBatch) <= 32764, "kernel parameter space");
+cudaError_t launch_finish_batch(FinishBatch& b, cudaStream_t s);
 // loss = fixed-order sum of n per-block loss partials (one warp); err gets
 // the non-finite bit
 cudaError_t launch_loss_reduce(const double* part, long long n, double* loss, int* err, cudaStream_t s);

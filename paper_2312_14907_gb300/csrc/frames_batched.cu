@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1) frames_batched(const __grid_
   cp_async_wait_all();
 }
 
-// One persistent launch over the frames of every problem with frame side M
-// (items are single frames); the block shape and occupancy are those of the
+// One persistent launch over the frames of every problem with frame side
+// M = 32 or 64 (items are single frames); the block shape and occupancy are those of the
 // single-problem kernel for M.  TMA: the inputs by tile and bulk copies as in
 // the single-problem kernel, each problem's objects through its own tensor
 // map (b.tmaps, device memory), on the block's mbarrier with the same bounded
@@ -156,7 +156,7 @@ bool batched_m_prepare(int m, bool tma, int* blocks_per_sm) {
     case 64:
       return tma ? prep(frames_batched_m<64, true>, T2Cfg<64>::T, T2Cfg<64>::SMEM_TMA)
                  : prep(frames_batched_m<64, false>, T2Cfg<64>::T, T2Cfg<64>::SMEM);
-    case 128: return !tma && prep(frames_batched_m<128, false>, T2Cfg<128>::T, T2Cfg<128>::SMEM);
+    case 128: return tma && batched128_prepare(blocks_per_sm);
     default: return false;
   }
 }
@@ -171,10 +171,7 @@ cudaError_t batched_m_launch(int m, bool tma, const BatchArgs& b, int grid, cuda
       if (tma) frames_batched_m<64, true><<<grid, T2Cfg<64>::T, T2Cfg<64>::SMEM_TMA, s>>>(b);
       else frames_batched_m<64, false><<<grid, T2Cfg<64>::T, T2Cfg<64>::SMEM, s>>>(b);
       break;
-    case 128:
-      if (tma) return cudaErrorInvalidValue;
-      frames_batched_m<128, false><<<grid, T2Cfg<128>::T, T2Cfg<128>::SMEM, s>>>(b);
-      break;
+    case 128: return tma ? batched128_launch(b, grid, s) : cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -40,8 +40,9 @@ struct BatchArgs {
                                          // tensor maps (device memory), else nullptr
   const int2* items;                     // [nitems] (problem, first frame)
   double* frame_part;                    // [frames][kBatchWarpSlots] loss partials,
-                                         // zeroed before the launch
-  int nitems;
+                                         // zeroed before the launch (side 128 on its
+                                         // own: [nprob][grid], every slot written)
+  int nitems;                            // (side 128 on its own: frames)
   int nprob;
 };
 
@@ -50,9 +51,13 @@ bool batched_prepare(int* blocks_per_sm);
 cudaError_t batched_launch(const BatchArgs& b, int grid, cudaStream_t s);
 
 // One launch per frame side: items are single frames of problems with side m.
-// tma (m = 32, 64): the inputs by tile and bulk copies, b.tmaps set.
+// tma (needed for m = 128): the inputs by tile and bulk copies, b.tmaps set.
+// m = 128: frame_base within the launch, each problem's frames in the order of
+// its FrameArgs::frames, no item table.
 bool batched_m_prepare(int m, bool tma, int* blocks_per_sm);
 cudaError_t batched_m_launch(int m, bool tma, const BatchArgs& b, int grid, cudaStream_t s);
+bool batched128_prepare(int* blocks_per_sm);
+cudaError_t batched128_launch(const BatchArgs& b, int grid, cudaStream_t s);
 
 // Layout of the M = 128 loss-and-gradient kernel (ignored for other sides):
 // radix-2 stages of each 128-point line across four threads by shuffles

@@ -570,57 +570,67 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
   tmem_fence_before_sync();
 }
 
-// loss and gradient (LOSS: loss only; FWD: the forward model; BG: with the
-// background of Eq. 2;
-// DET: the gradient through the deterministic plan p.det): a
-// persistent grid, block b taking frames [N b / G, N (b + 1) / G) of the
-// order given (p.frames, else 0..N-1); TMA: inputs by tile and bulk copies
-// (tm: the objects' tensor map), else by cp.async.  The probe values of a
-// thread sit in tensor memory and are reloaded when the frame's probe
-// changes: once per block for one probe, per peak for one probe per peak,
-// per frame for probes shifted per scan position.
-template <bool TMA, bool LOSS = false, bool BG = false, bool DET = false, bool FWD = false>
-__global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, const __grid_constant__ TmaMap tm) {
+// A block's shared state: buffers, barrier, tensor memory, twiddles.
+struct X3Block {
+  X3Roles r;
+  cf* buf;
+  float* abuf;
+  uint32_t tp, ta;       // the thread's lane: its probe words, the window's first column
+  uint32_t tmem;
+  BulkState bs;
+};
+
+// every thread of the block
+template <bool TMA>
+MPBP_DI void x3_begin(X3Block& b, unsigned char* smem_raw, uint64_t* mbar, uint32_t* tmem_base, X3Tables& tab) {
   using C = X3Cfg;
-  constexpr int M = C::M;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[C::T / 32];
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ uint32_t tmem_base;
-  __shared__ X3Tables tab;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && p.arrivals) *p.arrivals = 0u;
   unsigned char* smem = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
-  cf* buf = reinterpret_cast<cf*>(smem);
-  float* abuf = reinterpret_cast<float*>(smem + C::BUF);
-  const X3Roles r = X3Roles::make(threadIdx.x);
-  BulkState bs{smem_addr(&mbar), 0u, true};
+  b.buf = reinterpret_cast<cf*>(smem);
+  b.abuf = reinterpret_cast<float*>(smem + C::BUF);
+  b.r = X3Roles::make(threadIdx.x);
+  b.bs = BulkState{smem_addr(mbar), 0u, true};
   const int warp = threadIdx.x >> 5;
-  if (warp == 0) tmem_alloc(smem_addr(&tmem_base), C::TMEM_COLS);
-  if (TMA && threadIdx.x == 0) mbar_init(bs.bar, 1);
+  if (warp == 0) tmem_alloc(smem_addr(tmem_base), C::TMEM_COLS);
+  if (TMA && threadIdx.x == 0) mbar_init(b.bs.bar, 1);
   x3_tables_init(tab);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
+  b.tmem = *tmem_base;
   // this thread's lane is 32 (warp mod 4) + lane id = its column c; its probe
   // words are columns 64 (warp / 4) .. + 63; the window's slot s of column c
   // is columns 256 + 2 s, + 1 (every warp holding column c reaches them)
-  const uint32_t tp = tmem_addr(tmem_base, 32u * (warp & 3), 64u * (warp >> 2));
-  const uint32_t ta = tmem_addr(tmem_base, 32u * (warp & 3), C::ACC_COL);
+  b.tp = tmem_addr(b.tmem, 32u * (warp & 3), 64u * (warp >> 2));
+  b.ta = tmem_addr(b.tmem, 32u * (warp & 3), C::ACC_COL);
+}
+
+MPBP_DI void x3_end(const X3Block& b) {
+  tmem_fence_before_sync();
+  __syncthreads();
+  if ((threadIdx.x >> 5) == 0) tmem_dealloc(b.tmem, X3Cfg::TMEM_COLS);
+}
+
+// Frames [lo, hi) of the order given (p.frames, else 0..N-1) by one block;
+// returns the thread's share of the loss.  A wait that runs out clears
+// b.bs.ok and sets the error word.
+template <bool TMA, bool LOSS, bool BG, bool DET, bool FWD>
+MPBP_DI double x3_run(const FrameArgs& p, const TmaMap* tm, int lo, int hi, X3Block& b, const X3Tables& tab) {
+  using C = X3Cfg;
+  constexpr int M = C::M;
   if constexpr (!LOSS && !FWD) {
     // clear the window: warp w the slots 32 (w / 4) .. + 31 of its lanes
     const uint32_t z[16] = {};
-    sfor<0, 4>([&](auto k_) { tmem_st16(ta + 64u * (warp >> 2) + 16u * decltype(k_)::value, z); });
+    const int warp = threadIdx.x >> 5;
+    sfor<0, 4>([&](auto k_) { tmem_st16(b.ta + 64u * (warp >> 2) + 16u * decltype(k_)::value, z); });
     tmem_wait_st();
     tmem_fence_before_sync();   // ordered before the first frame's barriers
   }
   X3Win win{false, 0, 0, 0, DET ? p.det->block_piece0[blockIdx.x] - 1 : 0, INT_MAX, INT_MIN};
   const cf* tp_src = nullptr;   // the probe held in tensor memory (block-uniform)
   double lsum = 0.0;
-  const int lo = (int)((long long)p.nframes * blockIdx.x / gridDim.x);
-  const int hi = (int)((long long)p.nframes * (blockIdx.x + 1) / gridDim.x);
   const FrameRef none = frame_ref(p, p.nframes);   // not valid: nothing to fetch
   FrameRef cur = lo < hi ? frame_ref(p, lo) : none;
-  x3_fetch<TMA, FWD>(p, r, cur, buf, abuf, bs, &tm);
+  x3_fetch<TMA, FWD>(p, b.r, cur, b.buf, b.abuf, b.bs, tm);
   if constexpr (!TMA) cp_async_commit();
   // frame indices are read one frame ahead of their scan positions, so that
   // neither global load waits on the other
@@ -632,33 +642,58 @@ __global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, cons
     {
       const cf* P = frame_probe(p, cur, M * M);
       if (P != tp_src) {
-        x3_probe_to_tmem(P, r, tp);
+        x3_probe_to_tmem(P, b.r, b.tp);
         tp_src = P;
       }
     }
-    x3_frame<TMA, LOSS, BG, DET, FWD>(p, r, cur, nxt, [&](float fl) { lsum += (double)fl; }, bs, &tm, buf, abuf, tp, ta,
-                            tab, win);
-    if (TMA && !bs.ok) {
+    x3_frame<TMA, LOSS, BG, DET, FWD>(p, b.r, cur, nxt, [&](float fl) { lsum += (double)fl; }, b.bs, tm, b.buf, b.abuf,
+                                      b.tp, b.ta, tab, win);
+    if (TMA && !b.bs.ok) {
       if (threadIdx.x == 0) atomicOr(p.err, kErrTimeout);
       break;
     }
     cur = nxt;
   }
   cp_async_wait_all();
+  // the last frame announced a frame of no bytes after itself: its phase is
+  // complete, and the next run's first copies are the one after it
+  if (TMA && lo < hi) b.bs.parity ^= 1u;
   if constexpr (!LOSS && !FWD) {
-    if (bs.ok && win.ok) {   // what is left of the window
+    if (b.bs.ok && win.ok) {   // what is left of the window
       __syncthreads();
       tmem_fence_after_sync();
-      x3_flush<DET>(p, r, win, win.x, M, ta, false);
+      x3_flush<DET>(p, b.r, win, win.x, M, b.ta, false);
     }
   }
+  return lsum;
+}
+
+// loss and gradient (LOSS: loss only; FWD: the forward model; BG: with the
+// background of Eq. 2; DET: the gradient through the deterministic plan
+// p.det): a persistent grid, block b taking frames [N b / G, N (b + 1) / G)
+// of the order given; TMA: inputs by tile and bulk copies (tm: the objects'
+// tensor map), else by cp.async.  The probe values of a thread sit in tensor
+// memory and are reloaded when the frame's probe changes: once per block for
+// one probe, per peak for one probe per peak, per frame for probes shifted
+// per scan position.
+template <bool TMA, bool LOSS = false, bool BG = false, bool DET = false, bool FWD = false>
+__global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3(const FrameArgs p, const __grid_constant__ TmaMap tm) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[X3Cfg::T / 32];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tmem_base;
+  __shared__ X3Tables tab;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && p.arrivals) *p.arrivals = 0u;
+  X3Block b;
+  x3_begin<TMA>(b, smem_raw, &mbar, &tmem_base, tab);
+  const int lo = (int)((long long)p.nframes * blockIdx.x / gridDim.x);
+  const int hi = (int)((long long)p.nframes * (blockIdx.x + 1) / gridDim.x);
+  const double lsum = x3_run<TMA, LOSS, BG, DET, FWD>(p, &tm, lo, hi, b, tab);
   if constexpr (!FWD) {
-    const double tot = block_sum_d<C::T>(lsum, red);
+    const double tot = block_sum_d<X3Cfg::T>(lsum, red);
     if (threadIdx.x == 0) p.loss_part[blockIdx.x] = tot;
   }
-  tmem_fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem_base, C::TMEM_COLS);
+  x3_end(b);
 }
 
 }  // namespace mpbp

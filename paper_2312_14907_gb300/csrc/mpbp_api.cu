@@ -95,9 +95,10 @@ struct mpbp_ctx {
     BatchArgs args;
   };
   std::vector<PlanLaunch> batch_plan;
-  std::vector<long long> batch_base;  // first loss slot of each fused problem
   std::vector<int> batch_fused;       // batch positions of the fused problems
-  long long batch_frames = 0;
+  std::vector<std::pair<const double*, long long>> batch_loss;   // their loss partials
+  double* batch_part = nullptr;       // per-frame loss partials ...
+  long long batch_frames = 0;         // ... of this many frames, zeroed per call
   unsigned long long version = 0;     // bumped when probe or data change
   // lazily allocated for the host-buffer entry point: inputs, two staging
   // buffers for chunks of y, a copy stream and events for the pipeline
@@ -183,10 +184,11 @@ struct Carver {
   }
 };
 
-// whether problems of frame side m go through the batched kernel in `mode`
-bool batch_fused_side(int mode, int m) {
-  if (m < 32 || mode == 3) return false;
-  return mode != 2 || m < 128;
+// whether a problem goes through a batched kernel in `mode` (side 128 on its
+// own needs tile copies)
+bool batch_fused(int mode, const mpbp_ctx* c) {
+  if (c->M < 32 || mode == 3) return false;
+  return c->M < 128 || mode == 0 || (mode == 1 && c->tile_grad);
 }
 
 // frame-range launches of one host-path evaluation (each writes its own
@@ -478,9 +480,8 @@ mpbp_status enqueue_probe_shift(mpbp_ctx* c, cudaStream_t s) {
   return MPBP_OK;
 }
 
-mpbp_status enqueue_object_build(mpbp_ctx* c, const float* rho, const float* u,
-                                 const float* alpha, cf* out, cudaStream_t s,
-                                 const float* phi = nullptr, const AdamArgs* adam = nullptr) {
+ObjectArgs object_args(const mpbp_ctx* c, const float* rho, const float* u, const float* alpha, cf* out,
+                       const float* phi = nullptr, const AdamArgs* adam = nullptr) {
   ObjectArgs oa{};
   oa.rho = rho;
   oa.u = u;
@@ -494,7 +495,13 @@ mpbp_status enqueue_object_build(mpbp_ctx* c, const float* rho, const float* u,
   oa.C = c->C;
   oa.pc = c->pc;
   if (adam) oa.ad = *adam;
-  MPBP_CUDA(c, launch_object_build(oa, c->num_sms, s));
+  return oa;
+}
+
+mpbp_status enqueue_object_build(mpbp_ctx* c, const float* rho, const float* u,
+                                 const float* alpha, cf* out, cudaStream_t s,
+                                 const float* phi = nullptr, const AdamArgs* adam = nullptr) {
+  MPBP_CUDA(c, launch_object_build(object_args(c, rho, u, alpha, out, phi, adam), c->num_sms, s));
   return MPBP_OK;
 }
 
@@ -1663,13 +1670,13 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
     lead->batch_plan.clear();
     std::vector<int> fused;
     for (int i = 0; i < n; ++i)
-      if (batch_fused_side(lead->batch_mode, ctxs[i]->M)) fused.push_back(i);
+      if (batch_fused(lead->batch_mode, ctxs[i])) fused.push_back(i);
     const int nf = (int)fused.size();
     std::vector<long long> base(nf);
     long long total_frames = 0;
     for (int k = 0; k < nf; ++k) {
       base[k] = total_frames;
-      total_frames += ctxs[fused[k]]->nframes;
+      if (lead->batch_mode != 1 || ctxs[fused[k]]->M != 128) total_frames += ctxs[fused[k]]->nframes;
     }
     // frames per work item: a 256-thread block's worth in the single launch
     // over every side (mode 0), one frame in the per-side launches
@@ -1687,6 +1694,11 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
     auto add_launch = [&](int m, const std::vector<int>& probs) {
       Launch L{m, probs, items.size(), 0};
       const int np = (int)probs.size();
+      if (m == 128) {   // every problem's frames in its strip order: no items
+        for (int k : probs) L.count += (size_t)ctxs[fused[k]]->nframes;
+        if (L.count) launches.push_back(L);
+        return;
+      }
       for (int side : {128, 64, 32}) {
         if (lead->batch_order == 0) {
           for (int k = 0; k < np; ++k) {
@@ -1726,14 +1738,13 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
       if (!group.empty()) add_launch(side, group);
     }
     // device tables in the lead context's batch buffer
-    // per-side launches of frame sides 32 and 64 whose problems all have
-    // tile copies take their inputs by TMA, each
-    // problem through its own tensor map in the batch buffer
+    // per-side launches whose problems all have tile copies take their inputs
+    // by TMA, each problem through its own tensor map in the batch buffer
     std::vector<char> launch_tma(launches.size(), 0);
     size_t ntm = 0;
     for (size_t l = 0; l < launches.size(); ++l) {
       const Launch& L = launches[l];
-      if (L.m != 32 && L.m != 64) continue;
+      if (L.m == 0) continue;
       bool all = true;
       for (int k : L.probs) all = all && ctxs[fused[k]]->tile_grad;
       launch_tma[l] = all;
@@ -1743,6 +1754,7 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
     const size_t oI = cv.take<int2>(items.empty() ? 1 : items.size());
     const size_t oFP = cv.take<double>((size_t)(total_frames > 0 ? total_frames : 1) * kBatchWarpSlots);
     const size_t oTM = cv.take<TmaMap>(ntm > 0 ? ntm : 1);
+    const size_t oLP = cv.take<double>((size_t)(nf > 0 ? nf : 1) * lead->num_sms);   // side 128: [problem][block]
     const size_t need = align_up(cv.off, 256);
     if (need > lead->batch_ws_bytes) {
       MPBP_CUDA(lead, cudaStreamSynchronize(s));
@@ -1763,6 +1775,8 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
     double* frame_part = reinterpret_cast<double*>(wb + oFP);
     std::vector<TmaMap> tms(ntm > 0 ? ntm : 1);
     size_t tm_next = 0;
+    double* lp_next = reinterpret_cast<double*>(wb + oLP);
+    lead->batch_loss.assign((size_t)nf, {nullptr, 0});
     for (size_t l = 0; l < launches.size(); ++l) {
       const Launch& L = launches[l];
       mpbp_ctx::PlanLaunch P{};
@@ -1774,6 +1788,8 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
         P.args.probs[k] = frame_args(c, nullptr, (int)c->nframes);
         P.args.prob_m[k] = c->M;
         P.args.frame_base[k] = base[L.probs[k]];
+        lead->batch_loss[(size_t)L.probs[k]] = {frame_part + base[L.probs[k]] * kBatchWarpSlots,
+                                                c->nframes * kBatchWarpSlots};
         if (P.tma) {
           tms[tm_next] = c->tm_grad;
           tms[tm_next].tx_extra = c->test_tx_extra;
@@ -1788,35 +1804,48 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
       const bool ok = L.m == 0 ? batched_prepare(&bps) : batched_m_prepare(L.m, P.tma, &bps);
       if (!ok) return fail(lead, MPBP_ERR_CUDA, "batched kernel setup");
       P.grid = (int)std::min<long long>((long long)L.count, (long long)lead->num_sms * bps);
+      if (L.m == 128) {
+        long long f0 = 0;
+        for (size_t k = 0; k < L.probs.size(); ++k) {
+          mpbp_ctx* c = ctxs[fused[L.probs[k]]];
+          P.args.probs[k].frames = c->strip_order;
+          P.args.frame_base[k] = f0;
+          f0 += c->nframes;
+          lead->batch_loss[(size_t)L.probs[k]] = {lp_next + k * (size_t)P.grid, P.grid};
+        }
+        P.args.items = nullptr;
+        P.args.frame_part = lp_next;
+        lp_next += L.probs.size() * (size_t)P.grid;
+      }
       lead->batch_plan.push_back(P);
     }
     if (ntm > 0)
       MPBP_CUDA(lead, cudaMemcpyAsync(wb + oTM, tms.data(), sizeof(TmaMap) * ntm, cudaMemcpyHostToDevice, s));
-    lead->batch_base = base;
     lead->batch_fused = fused;
     lead->batch_frames = total_frames;
+    lead->batch_part = frame_part;
     lead->batch_key = key;
   }
-  const std::vector<long long>& base = lead->batch_base;
   const std::vector<int>& fused = lead->batch_fused;
   const int nf = (int)fused.size();
 
   // A1 for every problem
-  for (int i = 0; i < n; ++i) {
-    mpbp_ctx* c = ctxs[i];
-    if (c->acc_dirty) {
-      MPBP_CUDA(c, cudaMemsetAsync(c->acc, 0, sizeof(cf) * c->npix * c->D, s));
-      c->acc_dirty = false;
+  for (int i0 = 0; i0 < n; i0 += kAuxBatch) {
+    ObjectBatch ob;
+    ob.n = std::min(n - i0, kAuxBatch);
+    for (int k = 0; k < ob.n; ++k) {
+      mpbp_ctx* c = ctxs[i0 + k];
+      if (c->acc_dirty) {
+        MPBP_CUDA(c, cudaMemsetAsync(c->acc, 0, sizeof(cf) * c->npix * c->D, s));
+        c->acc_dirty = false;
+      }
+      ob.a[k] = object_args(c, rho[i0 + k], u[i0 + k], alpha[i0 + k], c->O);
     }
-    mpbp_status r = enqueue_object_build(c, rho[i], u[i], alpha[i], c->O, s);
-    if (r != MPBP_OK) return r;
+    MPBP_CUDA(lead, launch_object_build_batch(ob, lead->num_sms, s));
   }
   // A2..A7: the batched launches, then the usual kernel for M <= 16
-  double* frame_part = nullptr;
-  if (!lead->batch_plan.empty()) {
-    frame_part = lead->batch_plan[0].args.frame_part;
-    MPBP_CUDA(lead, cudaMemsetAsync(frame_part, 0, sizeof(double) * lead->batch_frames * kBatchWarpSlots, s));
-  }
+  if (lead->batch_frames > 0)
+    MPBP_CUDA(lead, cudaMemsetAsync(lead->batch_part, 0, sizeof(double) * lead->batch_frames * kBatchWarpSlots, s));
   for (int k = 0; k < nf; ++k) ctxs[fused[k]]->acc_dirty = true;
   for (const auto& P : lead->batch_plan) {
     if (P.m == 0) MPBP_CUDA(lead, batched_launch(P.args, P.grid, s));
@@ -1825,49 +1854,54 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
   std::vector<int> grid_of(n, 0);
   for (int i = 0; i < n; ++i) {
     mpbp_ctx* c = ctxs[i];
-    if (batch_fused_side(lead->batch_mode, c->M)) continue;
+    if (batch_fused(lead->batch_mode, c)) continue;
     FrameArgs fa = frame_args(c, nullptr, (int)c->nframes);
     grid_of[i] = frames_grid_for(c, c->nframes);
     c->acc_dirty = true;
     MPBP_CUDA(c, launch_frames(c, fa, grid_of[i], s));
   }
-  // A6/A7 tail and A8 reductions per problem
+  // A6/A7 tail and A8 reductions of every problem
   int k = 0;
-  for (int i = 0; i < n; ++i) {
-    mpbp_ctx* c = ctxs[i];
-    FinishArgs fi{};
-    fi.rho = rho[i];
-    fi.u = u[i];
-    fi.alpha = alpha[i];
-    fi.acc = c->acc;
-    fi.g_rho = g_rho[i];
-    fi.g_u = g_u[i];
-    fi.part = c->part;
-    fi.arrivals = c->arrivals;
-    fi.npix = c->npix;
-    fi.D = c->D;
-    fi.C = c->C;
-    fi.pc = c->pc;
-    ReduceArgs ra{};
-    if (batch_fused_side(lead->batch_mode, c->M)) {
-      fi.loss_part = frame_part + base[k] * kBatchWarpSlots;
-      fi.n_loss_part = c->nframes * kBatchWarpSlots;
-      ++k;
-    } else {
-      fi.loss_part = c->loss_part;
-      fi.n_loss_part = grid_of[i];
+  for (int i0 = 0; i0 < n; i0 += kAuxBatch) {
+    FinishBatch fb;
+    fb.n = std::min(n - i0, kAuxBatch);
+    for (int j = 0; j < fb.n; ++j) {
+      const int i = i0 + j;
+      mpbp_ctx* c = ctxs[i];
+      FinishArgs& fi = fb.a[j] = FinishArgs{};
+      fi.rho = rho[i];
+      fi.u = u[i];
+      fi.alpha = alpha[i];
+      fi.acc = c->acc;
+      fi.g_rho = g_rho[i];
+      fi.g_u = g_u[i];
+      fi.part = c->part;
+      fi.arrivals = c->arrivals;
+      fi.npix = c->npix;
+      fi.D = c->D;
+      fi.C = c->C;
+      fi.pc = c->pc;
+      if (batch_fused(lead->batch_mode, c)) {
+        fi.loss_part = lead->batch_loss[(size_t)k].first;
+        fi.n_loss_part = lead->batch_loss[(size_t)k].second;
+        ++k;
+      } else {
+        fi.loss_part = c->loss_part;
+        fi.n_loss_part = grid_of[i];
+      }
+      ReduceArgs& ra = fb.r[j] = ReduceArgs{};
+      ra.part = c->part;
+      ra.n_part = c->finish_grid;
+      ra.D = c->D;
+      ra.loss_out = loss[i];
+      ra.g_alpha_out = g_alpha ? g_alpha[i] : nullptr;
+      ra.g_alpha_ws = c->g_alpha_ws;
+      ra.err = c->err;
+      ra.st = nullptr;
+      ra.alpha_from = 1;
     }
-    ra.part = c->part;
-    ra.n_part = c->finish_grid;
-    ra.D = c->D;
-    ra.loss_out = loss[i];
-    ra.g_alpha_out = g_alpha ? g_alpha[i] : nullptr;
-    ra.g_alpha_ws = c->g_alpha_ws;
-    ra.err = c->err;
-    ra.st = nullptr;
-    ra.alpha_from = 1;
-    MPBP_CUDA(c, launch_finish(fi, ra, c->finish_grid, s));
-    c->acc_dirty = false;
+    MPBP_CUDA(lead, launch_finish_batch(fb, s));
+    for (int j = 0; j < fb.n; ++j) ctxs[i0 + j]->acc_dirty = false;
   }
   return MPBP_OK;
 }

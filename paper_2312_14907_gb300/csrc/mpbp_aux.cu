@@ -47,9 +47,10 @@ enum ObjectForm {
              // block 0 also counts the Adam step
 };
 
+// block bid of the nblk that work on a
 template <int FORM>
-__global__ void object_build_kernel(ObjectArgs a) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
+__device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int nblk) {
+  const long long stride = (long long)nblk * blockDim.x;
   const int pad = a.pitch - a.n2;
   const long long ostride = a.npix / a.n2 * a.pitch;
   __shared__ float s_alpha[kMaxPeaks];
@@ -58,7 +59,7 @@ __global__ void object_build_kernel(ObjectArgs a) {
     if constexpr (FORM == kObjAdam) s_alpha[m] = m == 0 ? 1.0f : expf(a.ad.alpha_t[m]);
     else s_alpha[m] = a.alpha[m];
   }
-  if (FORM == kObjAdam && blockIdx.x == 0) {
+  if (FORM == kObjAdam && bid == 0) {
     mpbp_adam_state* st = a.ad.st;
     const long long t = st->t + 1;
     __syncthreads();   // every thread has read the old count
@@ -69,7 +70,7 @@ __global__ void object_build_kernel(ObjectArgs a) {
     if (threadIdx.x == 32) st->bc2 = one_minus_pow(st->beta2, t);
   }
   __syncthreads();
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < a.npix; p += stride) {
+  for (long long p = (long long)bid * blockDim.x + threadIdx.x; p < a.npix; p += stride) {
     const long long q = pad ? p + (unsigned)p / (unsigned)a.n2 * (long long)pad : p;   // npix < 2^31
     float r;
     if constexpr (FORM == kObjAdam) r = (a.ad.mask ? a.ad.mask[p] : 1.0f) * expf(a.ad.chi[p]);
@@ -94,6 +95,26 @@ __global__ void object_build_kernel(ObjectArgs a) {
       }
     }
   }
+}
+
+template <int FORM>
+__global__ void object_build_kernel(const __grid_constant__ ObjectArgs a) {
+  object_build<FORM>(a, blockIdx.x, gridDim.x);
+}
+
+// Which of the n problems of a batched launch block b works on: block0[k] is
+// problem k's first block, block0[n] the grid.
+__device__ __forceinline__ int batch_problem(const int* block0, int n, int b) {
+  int k = 0;
+  while (k + 1 < n && b >= block0[k + 1]) ++k;
+  return k;
+}
+
+// The objects of several problems in one launch (16 problems of 128^2 to
+// 512^2: 16 launches of 4 us each became one).
+__global__ void object_build_batch_kernel(const __grid_constant__ ObjectBatch b) {
+  const int k = batch_problem(b.block0, b.n, blockIdx.x);
+  object_build<kObjU>(b.a[k], blockIdx.x - b.block0[k], b.block0[k + 1] - b.block0[k]);
 }
 
 // ----------------------------------------------------------------------------
@@ -376,8 +397,9 @@ __device__ __forceinline__ void adam_var(const AdamCoef& k, float lr, float g, f
   *xp = x - lr * (m * k.ic1) / (sqrtf(v * k.ic2) + k.eps);
 }
 
+// block bid of the nblk that work on a
 template <int FORM, int MP>
-__global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, ReduceArgs ra) {
+__device__ __forceinline__ void finish(const FinishArgs& a, const ReduceArgs& ra, int bid, int nblk) {
   constexpr bool STEP = FORM == kFinStep;
   constexpr int NW = kFinishThreads / 32;
   constexpr int NQ = MP + 3;
@@ -392,8 +414,8 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
 #pragma unroll
   for (int m = 0; m < MP; ++m) ap[m] = 0.f;
   float n_rho = 0.f, n_u = 0.f;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long p0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long stride = (long long)nblk * blockDim.x;
+  const long long p0 = (long long)bid * blockDim.x + threadIdx.x;
   // the frame kernel's loss partials (FP64), issued first: this block's
   // slice of them, or with STEP all of them in a fixed order
   double lp = 0.0;
@@ -543,7 +565,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
   }
   if (lane == 0) wsum[w][a.D + 2] = lp;
   __syncthreads();
-  double* out = a.part + (long long)blockIdx.x * (a.D + 3);
+  double* out = a.part + (long long)bid * (a.D + 3);
   if (w == 0 && lane < a.D + 3) {
     double t = 0.0;
 #pragma unroll
@@ -552,11 +574,26 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(FinishArgs a, Re
     __threadfence();   // publish this block's partials before counting it in
   }
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(a.arrivals, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) last = atomicAdd(a.arrivals, 1u) == (unsigned)nblk - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();
   final_reduce<kFinishThreads, FORM>(ra, STEP ? s_loss : 0.0);
+}
+
+template <int FORM, int MP>
+__global__ void __launch_bounds__(kFinishThreads)
+    finish_kernel(const __grid_constant__ FinishArgs a, const __grid_constant__ ReduceArgs ra) {
+  finish<FORM, MP>(a, ra, blockIdx.x, gridDim.x);
+}
+
+// The gradient assembly of several problems in one launch: each problem's
+// blocks reduce among themselves (its own arrival counter), as in a launch of
+// its own.
+template <int MP>
+__global__ void __launch_bounds__(kFinishThreads) finish_batch_kernel(const __grid_constant__ FinishBatch b) {
+  const int k = batch_problem(b.block0, b.n, blockIdx.x);
+  finish<kFinGrad, MP>(b.a[k], b.r[k], blockIdx.x - b.block0[k], b.block0[k + 1] - b.block0[k]);
 }
 
 // The loss alone (mpbp_loss): one warp sums the frame kernel's per-block
@@ -741,6 +778,14 @@ cudaError_t launch_object_build(const ObjectArgs& a, int num_sms, cudaStream_t s
   return cudaGetLastError();
 }
 
+cudaError_t launch_object_build_batch(ObjectBatch& b, int num_sms, cudaStream_t s) {
+  if (b.n < 1 || b.n > kAuxBatch) return cudaErrorInvalidValue;
+  b.block0[0] = 0;
+  for (int k = 0; k < b.n; ++k) b.block0[k + 1] = b.block0[k] + grid_for(b.a[k].npix, 256, num_sms * 8);
+  object_build_batch_kernel<<<b.block0[b.n], 256, 0, s>>>(b);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_counts16(const unsigned short* in, float* out, long long n, int num_sms, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   counts16_kernel<<<grid_for(n, 256, num_sms * 8), 256, 0, s>>>(in, out, n);
@@ -785,6 +830,21 @@ cudaError_t launch_finish(const FinishArgs& a, const ReduceArgs& r, int grid, cu
   if (a.phi) return launch_finish_form<kFinPhi>(a, r, grid, s);
   if (r.step.rho) return launch_finish_form<kFinStep>(a, r, grid, s);
   return launch_finish_form<kFinGrad>(a, r, grid, s);
+}
+
+cudaError_t launch_finish_batch(FinishBatch& b, cudaStream_t s) {
+  if (b.n < 1 || b.n > kAuxBatch) return cudaErrorInvalidValue;
+  int d = 0;
+  b.block0[0] = 0;
+  for (int k = 0; k < b.n; ++k) {
+    b.block0[k + 1] = b.block0[k] + b.r[k].n_part;   // one partial a block
+    d = std::max(d, b.a[k].D);
+  }
+  const int grid = b.block0[b.n];
+  if (d <= 4) finish_batch_kernel<4><<<grid, kFinishThreads, 0, s>>>(b);
+  else if (d <= 8) finish_batch_kernel<8><<<grid, kFinishThreads, 0, s>>>(b);
+  else finish_batch_kernel<kMaxPeaks><<<grid, kFinishThreads, 0, s>>>(b);
+  return cudaGetLastError();
 }
 
 }  // namespace mpbp
