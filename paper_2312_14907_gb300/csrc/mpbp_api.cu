@@ -1439,7 +1439,7 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
                o_p2 = cv.take<int>(nodes), o_o2 = cv.take<int>(nodes), o_hp = cv.take<int>(nodes),
                o_ho = cv.take<int>(nodes), o_mn = cv.take<int>(nodes),
                o_b = cv.take<unsigned long long>(nodes), o_ek = cv.take<unsigned long long>(2 * nodes),
-               o_f = cv.take<int>(3), o_bc = cv.take<unsigned>(2),
+               o_f = cv.take<int>(3), o_bc = cv.take<unsigned>(2), o_l = cv.take<int>(5 * c->D + 1),
                o_phi = cv.take<float>(nodes), o_w = cv.take<float>(nodes);
   void* b = nullptr;
   MPBP_CUDA(c, cudaStreamSynchronize(s));
@@ -1447,8 +1447,12 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
     cudaGetLastError();
     return fail(c, MPBP_ERR_OOM, "unwrap workspace");
   }
-  c->uw_buf = b;
   char* p = static_cast<char*>(b);
+  if (cudaMemset(p + o_l, 0, sizeof(int) * (5 * c->D + 1)) != cudaSuccess) {
+    cudaFree(b);
+    return fail(c, MPBP_ERR_CUDA, "unwrap workspace");
+  }
+  c->uw_buf = b;
   UnwrapArgs& a = c->uw;
   a.rel = reinterpret_cast<float*>(p + o_rel);
   a.parent = reinterpret_cast<int*>(p + o_p);
@@ -1463,6 +1467,9 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
   a.flags = reinterpret_cast<int*>(p + o_f);
   a.bar_count = reinterpret_cast<unsigned*>(p + o_bc);
   a.bar_gen = a.bar_count + 1;
+  a.lists = reinterpret_cast<int*>(p + o_l);
+  a.map_flags = a.lists + 2 * c->D;
+  a.need_global = a.map_flags + 3 * c->D;
   a.err = c->err;
   a.npix = c->npix;
   a.nodes = nodes;
@@ -1471,20 +1478,29 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
   int rounds = 2;
   while ((1ll << rounds) < nodes) ++rounds;
   a.max_rounds = rounds + 2;
+  a.max_blocks = unwrap_map_blocks();
   c->pj_phi = reinterpret_cast<float*>(p + o_phi);
   c->pj_wrapped = reinterpret_cast<float*>(p + o_w);
   return MPBP_OK;
 }
 
-mpbp_status enqueue_unwrap(mpbp_ctx* c, const float* wrapped, const float* mask, float* out, cudaStream_t s) {
+UnwrapArgs unwrap_args(const mpbp_ctx* c, const float* wrapped, const float* mask, float* out) {
   UnwrapArgs a = c->uw;
   a.wrapped = wrapped;
   a.mask = mask;
   a.out = out;
   a.test_stall = c->test_tx_extra != 0 ? 1 : 0;
+  return a;
+}
+
+mpbp_status enqueue_unwrap(mpbp_ctx* c, const UnwrapArgs& a, cudaStream_t s) {
+  if (unwrap_by_tiles(a)) {
+    MPBP_CUDA(c, unwrap_tiles_launch(a, c->uw_grid, s));
+    return MPBP_OK;
+  }
   MPBP_CUDA(c, cudaMemsetAsync(a.flags, 0, sizeof(int) * 3, s));
   MPBP_CUDA(c, cudaMemsetAsync(a.bar_count, 0, sizeof(unsigned) * 2, s));
-  MPBP_CUDA(c, unwrap_launch(a, c->uw_grid, s));
+  MPBP_CUDA(c, unwrap_launch(a, c->uw_grid, false, s));
   return MPBP_OK;
 }
 
@@ -1531,7 +1547,11 @@ mpbp_status mpbp_unwrap_phases(mpbp_ctx* c, const float* wrapped, const float* m
   cudaStream_t s = S(stream);
   mpbp_status r = unwrap_setup(c, s);
   if (r != MPBP_OK) return r;
-  return enqueue_unwrap(c, wrapped, mask, out, s);
+  const UnwrapArgs a = unwrap_args(c, wrapped, mask, out);
+  r = enqueue_unwrap(c, a, s);
+  if (r != MPBP_OK) return r;
+  if (unwrap_by_tiles(a)) MPBP_CUDA(c, unwrap_close_launch(a, c->num_sms, s));
+  return MPBP_OK;
 }
 
 mpbp_status mpbp_project_displacement(mpbp_ctx* c, float* u, const float* mask, void* stream) {
@@ -1556,9 +1576,10 @@ mpbp_status mpbp_project_displacement(mpbp_ctx* c, float* u, const float* mask, 
       pa.pinv_scaled[k * kMaxPeaks + m] = (float)(pinv[k * c->D + m] / c->phase_scale);
     }
   MPBP_CUDA(c, project_phase_launch(pa, c->num_sms, s));
-  r = enqueue_unwrap(c, c->pj_wrapped, mask, c->pj_wrapped, s);
+  const UnwrapArgs a = unwrap_args(c, c->pj_wrapped, mask, c->pj_wrapped);
+  r = enqueue_unwrap(c, a, s);
   if (r != MPBP_OK) return r;
-  MPBP_CUDA(c, project_correct_launch(pa, c->num_sms, s));
+  MPBP_CUDA(c, project_correct_launch(pa, a, unwrap_by_tiles(a), c->num_sms, s));
   return MPBP_OK;
 }
 

@@ -21,9 +21,18 @@
 // its lowest-numbered pixel keeps its wrapped value.  The D phase maps form
 // one graph with D disconnected parts.
 //
-// All of it runs in one cooperative launch (every block resident), with grid
-// barriers that are bounded in time: if one runs out, the block records
-// kErrTimeout and leaves, and the rest run out at their next barrier.
+// Two paths reach the same forest, offsets and output:
+//   - maps of at most 1,280 tiles (572^2 pixels): one kernel contracts the
+//     16 x 16 tiles (reliabilities and edge keys formed on the way) and lists
+//     the components and edges that are left; one cluster of 8 or 16 blocks
+//     per map runs the remaining rounds on those lists; the caller's closing
+//     kernel applies the offsets.  What bounds it is the chain of rounds (three
+//     256^2 maps: 119 us a projector call, against 237);
+//   - larger maps, and maps whose lists do not fit that cluster: one
+//     cooperative launch (every block resident), bound by its grid barriers
+//     (~5 us each, about 35 of them; three 256^2 maps: 226 us), which are
+//     bounded in time: if one runs out, the block records kErrTimeout and
+//     leaves, and the rest run out at their next barrier.
 #include <cmath>
 #include <climits>
 
@@ -85,8 +94,21 @@ __device__ bool grid_sync(UnwrapArgs& a) {
 
 __device__ __forceinline__ bool in_mask(const UnwrapArgs& a, long long r) { return !a.mask || a.mask[r] != 0.0f; }
 
-// reliability of node v: 1 / sqrt(H^2 + V^2 + D1^2 + D2^2) when all eight
-// neighbours are in the grid and the mask, else 0
+// reliability 1 / sqrt(H^2 + V^2 + D1^2 + D2^2) of a pixel from its 3 x 3
+// neighbourhood P(di, dj)
+template <typename Pix>
+__device__ __forceinline__ float reliability_of(Pix&& P) {
+  const float c = P(0, 0);
+  const float h = wrapf(P(0, -1) - c) - wrapf(c - P(0, 1));
+  const float vv = wrapf(P(-1, 0) - c) - wrapf(c - P(1, 0));
+  const float d1 = wrapf(P(-1, -1) - c) - wrapf(c - P(1, 1));
+  const float d2 = wrapf(P(-1, 1) - c) - wrapf(c - P(1, -1));
+  const float dd = sqrtf(h * h + vv * vv + d1 * d1 + d2 * d2);
+  return 1.0f / fmaxf(dd, 1e-30f);
+}
+
+// reliability of node v, when all eight neighbours are in the grid and the
+// mask, else 0
 __device__ float reliability(const UnwrapArgs& a, long long v) {
   const long long m = v / a.npix, r = v - m * a.npix;
   const int i = (int)(r / a.n2), j = (int)(r - (long long)i * a.n2);
@@ -95,14 +117,7 @@ __device__ float reliability(const UnwrapArgs& a, long long v) {
     for (int dj = -1; dj <= 1; ++dj)
       if (!in_mask(a, r + (long long)di * a.n2 + dj)) return 0.0f;
   const float* w = a.wrapped + m * a.npix;
-  auto P = [&](int ii, int jj) { return w[(long long)ii * a.n2 + jj]; };
-  const float c = P(i, j);
-  const float h = wrapf(P(i, j - 1) - c) - wrapf(c - P(i, j + 1));
-  const float vv = wrapf(P(i - 1, j) - c) - wrapf(c - P(i + 1, j));
-  const float d1 = wrapf(P(i - 1, j - 1) - c) - wrapf(c - P(i + 1, j + 1));
-  const float d2 = wrapf(P(i - 1, j + 1) - c) - wrapf(c - P(i + 1, j - 1));
-  const float dd = sqrtf(h * h + vv * vv + d1 * d1 + d2 * d2);
-  return 1.0f / fmaxf(dd, 1e-30f);
+  return reliability_of([&](int di, int dj) { return w[(long long)(i + di) * a.n2 + j + dj]; });
 }
 
 // the other end of edge e = 2 v + dir (dir 0: right, 1: down), or -1
@@ -136,10 +151,96 @@ __device__ __forceinline__ unsigned long long edge_key(float w, long long e) {
 constexpr int kTile = 16;
 static_assert(kTile * kTile == kUnwrapThreads, "one node per thread");
 
+// A tile's shared state: local root and offset of every node, its node
+// number, its phase, and the heaviest edge incident to each root.
+struct TileState {
+  int lp[kUnwrapThreads], lo[kUnwrapThreads], gid[kUnwrapThreads];
+  float wv[kUnwrapThreads];
+  unsigned long long bk[kUnwrapThreads];
+};
+
+// bk of every local root from the nodes' edges (0: none): kr, kd to the right
+// and down, inside the tile or leaving it, kl, ku to the left and up where
+// those leave the tile.  Every thread of the block; ends behind a barrier.
+__device__ __forceinline__ void tile_best(TileState& s, int t, bool r_in, bool d_in, unsigned long long kr,
+                                          unsigned long long kd, unsigned long long kl, unsigned long long ku) {
+  s.bk[t] = 0ull;
+  __syncthreads();
+  const int r = s.lp[t];
+  if (kr) {
+    const int rq = r_in ? s.lp[t + 1] : -1;
+    if (rq != r) {
+      atomicMax(&s.bk[r], kr);
+      if (rq >= 0) atomicMax(&s.bk[rq], kr);
+    }
+  }
+  if (kd) {
+    const int rq = d_in ? s.lp[t + kTile] : -1;
+    if (rq != r) {
+      atomicMax(&s.bk[r], kd);
+      if (rq >= 0) atomicMax(&s.bk[rq], kd);
+    }
+  }
+  if (kl) atomicMax(&s.bk[r], kl);
+  if (ku) atomicMax(&s.bk[r], ku);
+  __syncthreads();
+}
+
+// The Boruvka rounds of one tile (rows i0.., columns j0.. of a map whose nodes
+// start at base); in: the thread's node exists.  Returns whether bk holds the
+// heaviest edges of the final components.
+__device__ bool contract_tile(TileState& s, int t, bool in, int i0, int j0, int n2, long long base,
+                              unsigned long long kr, unsigned long long kd, unsigned long long kl,
+                              unsigned long long ku) {
+  const bool r_in = t % kTile + 1 < kTile, d_in = t / kTile + 1 < kTile;
+  int *lp = s.lp, *lo = s.lo, *gid = s.gid;
+  float* wv = s.wv;
+  unsigned long long* bk = s.bk;
+  for (int round = 0; round < 2 * kTile; ++round) {
+    tile_best(s, t, r_in, d_in, kr, kd, kl, ku);
+    const int r = lp[t];
+    // hooks of the roots whose heaviest edge stays inside the tile
+    int hook_p = -1, hook_o = 0;
+    if (in && r == t && bk[t] != 0ull) {
+      const long long e = 0xFFFFFFFFll - (long long)(bk[t] & 0xFFFFFFFFull);
+      const long long pg = (e >> 1) - base;   // the edge's first end, within the map
+      const int pi = (int)(pg / n2), pj = (int)(pg - (long long)pi * n2);
+      const int qi = pi + (int)(e & 1), qj = pj + (int)(1 - (e & 1));
+      if (pi >= i0 && pj >= j0 && qi < i0 + kTile && qj < j0 + kTile) {
+        const int pl = (pi - i0) * kTile + (pj - j0), ql = (qi - i0) * kTile + (qj - j0);
+        const bool p_in_r = lp[pl] == t;
+        const int lr = p_in_r ? pl : ql, ls = p_in_r ? ql : pl;
+        const int sr = lp[ls];
+        if (!(bk[sr] == bk[t] && gid[t] < gid[sr])) {   // the shared edge: sr hooks under t
+          const float d = (wv[lr] + kTwoPi * (float)lo[lr]) - (wv[ls] + kTwoPi * (float)lo[ls]);
+          hook_p = sr;
+          hook_o = -(int)floorf(d / kTwoPi + 0.5f);
+        }
+      }
+    }
+    if (!__syncthreads_or(hook_p >= 0)) return true;
+    if (hook_p >= 0) {
+      lp[t] = hook_p;
+      lo[t] = hook_o;
+    }
+    __syncthreads();
+    // pointer jumping to the roots (a forest of 256 nodes: at most 9 passes)
+    for (int jump = 0; jump < 2 * kTile; ++jump) {
+      const int p = lp[t], pp = lp[p];
+      const int no = lo[t] + (pp != p ? lo[p] : 0);
+      __syncthreads();
+      if (pp != p) {
+        lp[t] = pp;
+        lo[t] = no;
+      }
+      if (!__syncthreads_or(pp != p)) break;
+    }
+  }
+  return false;
+}
+
 __device__ void local_contract(const UnwrapArgs& a) {
-  __shared__ int lp[kUnwrapThreads], lo[kUnwrapThreads], gid[kUnwrapThreads];
-  __shared__ float wv[kUnwrapThreads];
-  __shared__ unsigned long long bk[kUnwrapThreads];
+  __shared__ TileState s;
   const int t = threadIdx.x, ti = t / kTile, tj = t % kTile;
   const int n1 = a.n1, n2 = a.n2;
   const int tpr = (n2 + kTile - 1) / kTile, tpc = (n1 + kTile - 1) / kTile;
@@ -161,78 +262,294 @@ __device__ void local_contract(const UnwrapArgs& a) {
       if (tj == 0 && j > 0) kl = a.ekey[2 * (v - 1)];
       if (ti == 0 && i > 0) ku = a.ekey[2 * (v - n2) + 1];
     }
-    const bool r_in = tj + 1 < kTile, d_in = ti + 1 < kTile;
-    gid[t] = (int)v;
-    lp[t] = t;
-    lo[t] = 0;
-    wv[t] = in ? a.wrapped[v] : 0.0f;
-    for (int round = 0; round < 2 * kTile; ++round) {
-      bk[t] = 0ull;
-      __syncthreads();
-      const int r = lp[t];
-      if (kr) {
-        const int rq = r_in ? lp[t + 1] : -1;
-        if (rq != r) {
-          atomicMax(&bk[r], kr);
-          if (rq >= 0) atomicMax(&bk[rq], kr);
-        }
-      }
-      if (kd) {
-        const int rq = d_in ? lp[t + kTile] : -1;
-        if (rq != r) {
-          atomicMax(&bk[r], kd);
-          if (rq >= 0) atomicMax(&bk[rq], kd);
-        }
-      }
-      if (kl) atomicMax(&bk[r], kl);
-      if (ku) atomicMax(&bk[r], ku);
-      __syncthreads();
-      // hooks of the roots whose heaviest edge stays inside the tile
-      int hook_p = -1, hook_o = 0;
-      if (in && r == t && bk[t] != 0ull) {
-        const long long e = 0xFFFFFFFFll - (long long)(bk[t] & 0xFFFFFFFFull);
-        const long long pg = (e >> 1) - base;   // the edge's first end, within the map
-        const int pi = (int)(pg / n2), pj = (int)(pg - (long long)pi * n2);
-        const int qi = pi + (int)(e & 1), qj = pj + (int)(1 - (e & 1));
-        if (pi >= i0 && pj >= j0 && qi < i0 + kTile && qj < j0 + kTile) {
-          const int pl = (pi - i0) * kTile + (pj - j0), ql = (qi - i0) * kTile + (qj - j0);
-          const bool p_in_r = lp[pl] == t;
-          const int lr = p_in_r ? pl : ql, ls = p_in_r ? ql : pl;
-          const int sr = lp[ls];
-          if (!(bk[sr] == bk[t] && gid[t] < gid[sr])) {   // the shared edge: sr hooks under t
-            const float d = (wv[lr] + kTwoPi * (float)lo[lr]) - (wv[ls] + kTwoPi * (float)lo[ls]);
-            hook_p = sr;
-            hook_o = -(int)floorf(d / kTwoPi + 0.5f);
-          }
-        }
-      }
-      if (!__syncthreads_or(hook_p >= 0)) break;
-      if (hook_p >= 0) {
-        lp[t] = hook_p;
-        lo[t] = hook_o;
-      }
-      __syncthreads();
-      // pointer jumping to the roots (a forest of 256 nodes: at most 9 passes)
-      for (int jump = 0; jump < 2 * kTile; ++jump) {
-        const int p = lp[t], pp = lp[p];
-        const int no = lo[t] + (pp != p ? lo[p] : 0);
-        __syncthreads();
-        if (pp != p) {
-          lp[t] = pp;
-          lo[t] = no;
-        }
-        if (!__syncthreads_or(pp != p)) break;
-      }
-    }
+    s.gid[t] = (int)v;
+    s.lp[t] = t;
+    s.lo[t] = 0;
+    s.wv[t] = in ? a.wrapped[v] : 0.0f;
+    contract_tile(s, t, in, i0, j0, n2, base, kr, kd, kl, ku);
     if (in) {
-      a.parent[v] = gid[lp[t]];
-      a.off[v] = lo[t];
+      a.parent[v] = s.gid[s.lp[t]];
+      a.off[v] = s.lo[t];
     }
     __syncthreads();   // the next tile reuses the shared arrays
   }
 }
 
-__global__ void __launch_bounds__(kUnwrapThreads) unwrap_kernel(UnwrapArgs a) {
+// ----------------------------------------------------------------------------
+// The path by tiles and maps.  Arrays of UnwrapArgs in other roles:
+//   parent, off       tile-local root and offset of every node
+//   parent2[root]     the component's label in its map, or -1 where no edge
+//                     leaves it
+//   off2[root]        what is added to off for the output
+//   of component l of a map (at the map's first node + l): hook_off its root,
+//   minnode its lowest node, hook_parent that node's off
+//   ekey              per map, npix / 2 listed edges' keys, then npix / 2
+//                     places each for the components' parent and offset (two
+//                     buffers), hook and hook offset
+//   best              of component l of a map, as everywhere
+//   lists[2 m]        components and edges listed (zero between calls)
+// ----------------------------------------------------------------------------
+
+__device__ __forceinline__ int map_cap(const UnwrapArgs& a) { return (int)(a.npix / 2); }   // components, edges
+__device__ __forceinline__ unsigned long long* map_keys(const UnwrapArgs& a, int m) { return a.ekey + 2 * m * a.npix; }
+
+// one block per tile: reliabilities, edge keys, contraction, lists
+__global__ void __launch_bounds__(kUnwrapThreads) unwrap_tile_kernel(UnwrapArgs a) {
+  constexpr int W = kTile + 4, R = kTile + 2;
+  __shared__ TileState s;
+  __shared__ float sw[W * W], srel[R * R];
+  __shared__ unsigned char sin[W * W];   // in the grid and the mask
+  __shared__ int lmin[kUnwrapThreads], s_n[2], s_at[2];
+  const int t = threadIdx.x, ti = t / kTile, tj = t % kTile;
+  const int n1 = a.n1, n2 = a.n2;
+  const int tpr = (n2 + kTile - 1) / kTile, tpc = (n1 + kTile - 1) / kTile;
+  const int m = blockIdx.x / (tpr * tpc), rem = blockIdx.x - m * (tpr * tpc);
+  const int i0 = rem / tpr * kTile, j0 = rem % tpr * kTile;
+  const long long base = (long long)m * a.npix;
+  if (blockIdx.x == 0 && t < 6) {   // for the cooperative kernel that may follow
+    if (t < 3) a.flags[t] = 0;
+    else if (t < 5) a.bar_count[t - 3] = 0u;
+    else *a.need_global = 0;
+  }
+  for (int k = t; k < W * W; k += kUnwrapThreads) {
+    const int i = i0 - 2 + k / W, j = j0 - 2 + k % W;
+    const bool ok = i >= 0 && j >= 0 && i < n1 && j < n2 && in_mask(a, (long long)i * n2 + j);
+    sin[k] = ok;
+    sw[k] = ok ? a.wrapped[base + (long long)i * n2 + j] : 0.0f;
+  }
+  if (t < 2) s_n[t] = 0;
+  __syncthreads();
+  for (int k = t; k < R * R; k += kUnwrapThreads) {
+    const int c = (k / R + 1) * W + k % R + 1;
+    bool all = true;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) all = all && sin[c + (q / 3 - 1) * W + q % 3 - 1];
+    srel[k] = all ? reliability_of([&](int di, int dj) { return sw[c + di * W + dj]; }) : 0.0f;
+  }
+  __syncthreads();
+  const int i = i0 + ti, j = j0 + tj;
+  const bool in = i < n1 && j < n2;
+  const long long v = in ? base + (long long)i * n2 + j : -1;
+  const int c = (ti + 2) * W + tj + 2, q = (ti + 1) * R + tj + 1;
+  unsigned long long kr = 0, kd = 0, kl = 0, ku = 0;
+  if (in && sin[c]) {
+    if (sin[c + 1]) kr = edge_key(srel[q] + srel[q + 1], 2 * v);
+    if (sin[c + W]) kd = edge_key(srel[q] + srel[q + R], 2 * v + 1);
+    if (tj == 0 && sin[c - 1]) kl = edge_key(srel[q - 1] + srel[q], 2 * (v - 1));
+    if (ti == 0 && sin[c - W]) ku = edge_key(srel[q - R] + srel[q], 2 * (v - n2) + 1);
+  }
+  s.gid[t] = (int)v;
+  s.lp[t] = t;
+  s.lo[t] = 0;
+  // (a pixel off the mask has no edges: its phase is not read)
+  s.wv[t] = sw[c];
+  const bool r_in = tj + 1 < kTile, d_in = ti + 1 < kTile;
+  if (!contract_tile(s, t, in, i0, j0, n2, base, kr, kd, kl, ku)) tile_best(s, t, r_in, d_in, kr, kd, kl, ku);
+  // lists: the components that an edge leaves, and those edges, each by the
+  // tile of its first end
+  lmin[t] = kUnwrapThreads;
+  __syncthreads();
+  const int root = s.lp[t];
+  if (in) atomicMin(&lmin[root], t);   // t grows with the node number
+  const bool listed = in && root == t && s.bk[t] != 0ull;
+  const bool er = kr && !(r_in && s.lp[t + 1] == root), ed = kd && !(d_in && s.lp[t + kTile] == root);
+  const int lc = listed ? atomicAdd(&s_n[0], 1) : 0;
+  const int le = er || ed ? atomicAdd(&s_n[1], (int)er + (int)ed) : 0;
+  __syncthreads();
+  if (t < 2) s_at[t] = s_n[t] ? atomicAdd(&a.lists[2 * m + t], s_n[t]) : 0;
+  __syncthreads();
+  if (in) {
+    a.parent[v] = s.gid[root];
+    a.off[v] = s.lo[t];
+    if (root == t) {
+      const int lm = lmin[t];
+      if (listed) {
+        const int l = s_at[0] + lc;
+        a.parent2[v] = l;
+        a.hook_off[base + l] = (int)v;
+        a.minnode[base + l] = s.gid[lm];
+        a.hook_parent[base + l] = s.lo[lm];
+      } else {
+        a.parent2[v] = -1;
+        a.off2[v] = -s.lo[lm];
+      }
+    }
+    const int k = s_at[1] + le, cap = map_cap(a);   // past it, the map kernel gives the work up
+    unsigned long long* const ek = map_keys(a, m);
+    if (er && k < cap) ek[k] = kr;
+    if (ed && k + er < cap) ek[k + er] = kd;
+  }
+}
+
+// A map's cluster: threads a block, edges a thread keeps in registers.
+constexpr int kMapThreads = 1024;
+constexpr int kMapEdges = 8;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// One cluster per map: the remaining rounds on the listed components and
+// edges, in L2, with the cluster's hardware barrier (about 1 us a phase with
+// the reads around it, against 5 us for the grid's; one block instead of
+// eight, its state in shared memory, took longer than the whole grid: it is
+// bound by its SM's issue and by one lane a clock for its scattered reads).
+__global__ void __launch_bounds__(kMapThreads) unwrap_map_kernel(UnwrapArgs a, int blocks) {
+  const int m = blockIdx.x / blocks;
+  const int t = (blockIdx.x % blocks) * kMapThreads + threadIdx.x;   // within the cluster
+  const int all = blocks * kMapThreads;
+  const long long base = (long long)m * a.npix;
+  const int cap = map_cap(a);
+  const int nc = a.lists[2 * m], ne = a.lists[2 * m + 1];
+  if (nc > cap || ne > cap || ne > (long long)all * kMapEdges) {   // the cooperative kernel starts over
+    if (t == 0) *a.need_global = 1;
+    return;
+  }
+  const unsigned long long* const ek = map_keys(a, m);
+  int* const pool = reinterpret_cast<int*>(map_keys(a, m) + cap);
+  int* const par[2] = {pool, pool + cap};
+  int* const off[2] = {pool + 2 * cap, pool + 3 * cap};
+  int* const hp = pool + 4 * cap;
+  int* const ho = pool + 5 * cap;
+  unsigned long long* const best = a.best + base;
+  int* const flags = a.map_flags + 3 * m;   // rotating: the next slot is cleared two uses after its last read
+  int use = 0, cur = 0;
+  auto label = [&](long long v) { return a.parent2[a.parent[v]]; };
+  auto ends = [&](unsigned long long key, long long& p, long long& q) {
+    const long long e = 0xFFFFFFFFll - (long long)(key & 0xFFFFFFFFull);
+    p = e >> 1;
+    q = p + ((e & 1) ? a.n2 : 1);
+  };
+  for (int l = t; l < nc; l += all) {
+    par[0][l] = l;
+    off[0][l] = 0;
+    best[l] = 0ull;
+  }
+  if (t < 3) flags[t] = 0;
+  unsigned long long key[kMapEdges];   // 0: none, or inside a component
+  int la[kMapEdges], lb[kMapEdges];
+#pragma unroll
+  for (int i = 0; i < kMapEdges; ++i) {
+    const int k = t + i * all;
+    key[i] = k < ne ? ek[k] : 0ull;
+    la[i] = lb[i] = 0;
+    if (key[i]) {
+      long long p, q;
+      ends(key[i], p, q);
+      la[i] = label(p);
+      lb[i] = label(q);
+    }
+  }
+  cluster_sync();
+  for (int round = 0; round < a.max_rounds; ++round) {
+    // heaviest incident edge of every component
+#pragma unroll
+    for (int i = 0; i < kMapEdges; ++i) {
+      if (!key[i]) continue;
+      la[i] = __ldcg(par[cur] + la[i]);   // the components the ends are in by now
+      lb[i] = __ldcg(par[cur] + lb[i]);
+      if (la[i] == lb[i]) {
+        key[i] = 0ull;
+        continue;
+      }
+      if (key[i] > __ldcg(best + la[i])) atomicMax(best + la[i], key[i]);
+      if (key[i] > __ldcg(best + lb[i])) atomicMax(best + lb[i], key[i]);
+    }
+    cluster_sync();
+    const int fs = use % 3;
+    for (int l = t; l < nc; l += all) {
+      const unsigned long long b = __ldcg(best + l);
+      int h = -1;
+      if (b != 0ull) {   // a root: nothing else has one
+        long long p, q;
+        ends(b, p, q);
+        const int lp = label(p), lq = label(q);
+        const bool p_in = __ldcg(par[cur] + lp) == l;
+        const int s = __ldcg(par[cur] + (p_in ? lq : lp));
+        if (!(__ldcg(best + s) == b && a.hook_off[base + l] < a.hook_off[base + s])) {   // else s hooks under l
+          const float dp = a.wrapped[p] + kTwoPi * (float)(a.off[p] + __ldcg(off[cur] + lp));
+          const float dq = a.wrapped[q] + kTwoPi * (float)(a.off[q] + __ldcg(off[cur] + lq));
+          const float d = p_in ? dp - dq : dq - dp;
+          h = s;
+          ho[l] = -(int)floorf(d / kTwoPi + 0.5f);
+          flags[fs] = 1;
+        }
+      }
+      hp[l] = h;
+    }
+    if (t == 0) flags[(use + 1) % 3] = 0;
+    cluster_sync();
+    const bool any = __ldcg(flags + fs) != 0;
+    ++use;
+    if (!any) break;
+    // pointer jumping, four hops a pass, until every component is under a
+    // root; the first pass applies the hooks and clears best (the cap only
+    // guards against a forest that is not one)
+    for (int jump = 0; jump < 32; ++jump) {
+      const int fj = use % 3;
+      auto up = [&](int x, int& o) {
+        if (jump == 0) {
+          const int h = __ldcg(hp + x);
+          if (h >= 0) {
+            o = __ldcg(ho + x);
+            return h;
+          }
+        }
+        o = __ldcg(off[cur] + x);
+        return __ldcg(par[cur] + x);
+      };
+      for (int l = t; l < nc; l += all) {
+        int o = 0, sum = 0, x = l;
+#pragma unroll
+        for (int hop = 0; hop < 4; ++hop) {
+          const int y = up(x, o);
+          sum += o;   // a root's is 0
+          if (y == x) break;
+          x = y;
+        }
+        par[cur ^ 1][l] = x;
+        off[cur ^ 1][l] = sum;
+        if (up(x, o) != x) flags[fj] = 1;
+        if (jump == 0) best[l] = 0ull;
+      }
+      if (t == 0) flags[(use + 1) % 3] = 0;
+      cluster_sync();
+      const bool more = __ldcg(flags + fj) != 0;
+      ++use;
+      cur ^= 1;
+      if (!more) break;
+    }
+  }
+  // each group's lowest-numbered node keeps its wrapped value
+  for (int l = t; l < nc; l += all) hp[l] = INT_MAX;
+  cluster_sync();
+  for (int l = t; l < nc; l += all) atomicMin(hp + __ldcg(par[cur] + l), a.minnode[base + l]);
+  cluster_sync();
+  for (int l = t; l < nc; l += all) {
+    const int r = __ldcg(par[cur] + l);
+    if (a.minnode[base + l] == __ldcg(hp + r)) ho[r] = a.hook_parent[base + l] + __ldcg(off[cur] + l);
+  }
+  cluster_sync();
+  for (int l = t; l < nc; l += all)
+    a.off2[a.hook_off[base + l]] = __ldcg(off[cur] + l) - __ldcg(ho + __ldcg(par[cur] + l));
+}
+
+// the unwrapped phase of node v after the tile and map kernels
+__device__ __forceinline__ float unwrapped_at(const UnwrapArgs& a, long long v) {
+  return a.wrapped[v] + kTwoPi * (float)(a.off[v] + a.off2[a.parent[v]]);
+}
+
+__global__ void unwrap_close_kernel(UnwrapArgs a, int maps) {
+  if (blockIdx.x == 0 && threadIdx.x < 2 * maps) a.lists[threadIdx.x] = 0;
+  if (*a.need_global) return;   // the cooperative kernel has written out
+  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.nodes;
+       v += (long long)gridDim.x * blockDim.x)
+    a.out[v] = unwrapped_at(a, v);
+}
+
+// The cooperative path; opt: only if the map kernel asked for it.
+__global__ void __launch_bounds__(kUnwrapThreads) unwrap_kernel(UnwrapArgs a, int opt) {
+  if (opt && *a.need_global == 0) return;
   const long long n = a.nodes;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -376,14 +693,22 @@ __global__ void project_phase_kernel(ProjectArgs a) {
   }
 }
 
-// u += (Phi' - Phi) pinv^T / phase_scale inside the mask
-__global__ void project_correct_kernel(ProjectArgs a) {
+// u += (Phi' - Phi) pinv^T / phase_scale inside the mask; tiles: Phi' from the
+// tile and map kernels' offsets, unless the cooperative kernel ran
+__global__ void project_correct_kernel(ProjectArgs a, UnwrapArgs uw, int tiles) {
+  if (tiles) {
+    if (blockIdx.x == 0 && threadIdx.x < 2 * a.D) uw.lists[threadIdx.x] = 0;
+    tiles = *uw.need_global == 0;
+  }
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < a.npix;
        r += (long long)gridDim.x * blockDim.x) {
     if (a.mask && a.mask[r] == 0.0f) continue;
     for (int c = 0; c < a.C; ++c) {
       float s = 0.0f;
-      for (int m = 0; m < a.D; ++m) s = fmaf(a.pinv_scaled[c * kMaxPeaks + m], a.unwrapped[m * a.npix + r] - a.phi[m * a.npix + r], s);
+      for (int m = 0; m < a.D; ++m) {
+        const long long i = m * a.npix + r;
+        s = fmaf(a.pinv_scaled[c * kMaxPeaks + m], (tiles ? unwrapped_at(uw, i) : a.unwrapped[i]) - a.phi[i], s);
+      }
       a.u[c * a.npix + r] += s;
     }
   }
@@ -400,8 +725,66 @@ bool unwrap_prepare(int num_sms, int* grid) {
   return true;
 }
 
-cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, cudaStream_t s) {
-  void* args[] = {const_cast<UnwrapArgs*>(&a)};
+// The map kernel's launch: `maps` clusters of `blocks` blocks.
+static cudaLaunchConfig_t map_config(int maps, int blocks, cudaLaunchAttribute* at, cudaStream_t s) {
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = (unsigned)blocks;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)(maps * blocks));
+  c.blockDim = dim3(kMapThreads);
+  c.stream = s;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return c;
+}
+
+int unwrap_map_blocks() {
+  cudaLaunchAttribute at;
+  int n = 0;
+  const cudaLaunchConfig_t c = map_config(1, 16, &at, nullptr);
+  if (cudaFuncSetAttribute(unwrap_map_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, unwrap_map_kernel, &c) == cudaSuccess && n > 0)
+    return 16;
+  cudaGetLastError();
+  return 8;
+}
+
+static long long map_tiles(const UnwrapArgs& a) {
+  return (long long)((a.n1 + kTile - 1) / kTile) * ((a.n2 + kTile - 1) / kTile);
+}
+
+// A tile leaves about 13 components and 85 edges on a noisy map (a pixel's
+// heaviest edge often leaves its tile): eight blocks hold the edges of 640
+// such tiles (404^2 pixels), sixteen those of 1,280 (572^2).
+constexpr long long kTilesPerBlock = 80;
+
+static int map_blocks(const UnwrapArgs& a) { return map_tiles(a) <= 8 * kTilesPerBlock ? 8 : 16; }
+
+bool unwrap_by_tiles(const UnwrapArgs& a) {
+  return !a.test_stall && map_tiles(a) <= a.max_blocks * kTilesPerBlock;
+}
+
+cudaError_t unwrap_tiles_launch(const UnwrapArgs& a, int grid, cudaStream_t s) {
+  const int maps = (int)(a.nodes / a.npix);
+  unwrap_tile_kernel<<<(unsigned)(map_tiles(a) * maps), kUnwrapThreads, 0, s>>>(a);
+  cudaLaunchAttribute at;
+  const int blocks = map_blocks(a);
+  const cudaLaunchConfig_t c = map_config(maps, blocks, &at, s);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&c, unwrap_map_kernel, a, blocks);
+  return e != cudaSuccess ? e : unwrap_launch(a, grid, true, s);
+}
+
+cudaError_t unwrap_close_launch(const UnwrapArgs& a, int num_sms, cudaStream_t s) {
+  const long long b = (a.nodes + 255) / 256;
+  unwrap_close_kernel<<<(int)(b < num_sms * 8 ? b : num_sms * 8), 256, 0, s>>>(a, (int)(a.nodes / a.npix));
+  return cudaGetLastError();
+}
+
+cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, bool optional, cudaStream_t s) {
+  int opt = optional ? 1 : 0;
+  void* args[] = {const_cast<UnwrapArgs*>(&a), &opt};
   return cudaLaunchCooperativeKernel((const void*)unwrap_kernel, dim3(grid), dim3(kUnwrapThreads), args, 0, s);
 }
 
@@ -412,9 +795,10 @@ cudaError_t project_phase_launch(const ProjectArgs& a, int num_sms, cudaStream_t
   return cudaGetLastError();
 }
 
-cudaError_t project_correct_launch(const ProjectArgs& a, int num_sms, cudaStream_t s) {
+cudaError_t project_correct_launch(const ProjectArgs& a, const UnwrapArgs& uw, bool tiles, int num_sms,
+                                   cudaStream_t s) {
   const long long b = (a.npix + 255) / 256;
-  project_correct_kernel<<<(int)(b < num_sms * 8 ? b : num_sms * 8), 256, 0, s>>>(a);
+  project_correct_kernel<<<(int)(b < num_sms * 8 ? b : num_sms * 8), 256, 0, s>>>(a, uw, tiles ? 1 : 0);
   return cudaGetLastError();
 }
 

@@ -4,7 +4,7 @@
 
 namespace mpbp {
 
-// one cooperative launch over D maps of n1 x n2 pixels (nodes = D * npix)
+// D maps of n1 x n2 pixels (nodes = D * npix)
 struct UnwrapArgs {
   const float* wrapped;   // [nodes] wrapped phases in [-pi, pi)
   const float* mask;      // [npix] nonzero = inside, or nullptr
@@ -22,10 +22,14 @@ struct UnwrapArgs {
   int* flags;             // [3] rotating "something changed" flags, zeroed before launch
   unsigned* bar_count;    // grid barrier, zeroed before launch
   unsigned* bar_gen;
+  int* lists;             // [2 D] components and edges listed per map, zero between calls
+  int* map_flags;         // [3 D] the map kernel's "something changed" flags
+  int* need_global;       // the map kernel leaves the work to the cooperative one
   int* err;               // kErrTimeout if a barrier wait runs out
   long long npix, nodes;
   int n1, n2;
   int max_rounds;
+  int max_blocks;         // largest cluster the map kernel may use (unwrap_map_blocks)
   int test_stall;         // != 0: block 0 never arrives at a grid barrier (test
                           // of the bounded waits; the result is meaningless)
 };
@@ -43,8 +47,20 @@ struct ProjectArgs {
 };
 
 bool unwrap_prepare(int num_sms, int* grid);
-cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, cudaStream_t s);
+int unwrap_map_blocks();
+// The cooperative path, on the given grid (optional: returns at once unless
+// *need_global); flags and barrier zeroed before.
+cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, bool optional, cudaStream_t s);
+// Whether the path by tiles and maps serves these maps; it, with the
+// cooperative launch behind it where a map leaves too many components; and
+// the kernel that writes out (project_correct does without).
+bool unwrap_by_tiles(const UnwrapArgs& a);
+cudaError_t unwrap_tiles_launch(const UnwrapArgs& a, int grid, cudaStream_t s);
+cudaError_t unwrap_close_launch(const UnwrapArgs& a, int num_sms, cudaStream_t s);
 cudaError_t project_phase_launch(const ProjectArgs& a, int num_sms, cudaStream_t s);
-cudaError_t project_correct_launch(const ProjectArgs& a, int num_sms, cudaStream_t s);
+// tiles: the unwrapped phases from uw's offsets (unwrap_tiles_launch without
+// unwrap_close_launch), else from a.unwrapped
+cudaError_t project_correct_launch(const ProjectArgs& a, const UnwrapArgs& uw, bool tiles, int num_sms,
+                                   cudaStream_t s);
 
 }  // namespace mpbp
