@@ -193,26 +193,30 @@ def load(build_if_missing=True):
     return lib
 
 
+# A call's marshalling runs on the host once per launch sequence, and at the
+# smallest problems (147 frames of 32 x 32, 20 us of kernels) it is what the
+# call takes.  So pointers and the stream go to ctypes as plain integers (the
+# argument types convert them), the stream comes from torch's raw getter
+# (current_stream() builds a Stream object), shapes are kept as tuples, and a
+# tensor that passes its checks goes through one expression.
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _p(t):
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _dev(t, dtype, shape, name):
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.shape == shape and t.is_contiguous():
+        return t
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError("%s must be a CUDA tensor" % name)
     if t.dtype != dtype:
         raise TypeError("%s must be %s, got %s" % (name, dtype, t.dtype))
     if tuple(t.shape) != tuple(shape):
         raise ValueError("%s must have shape %s, got %s" % (name, tuple(shape), tuple(t.shape)))
-    if not t.is_contiguous():
-        raise ValueError("%s must be contiguous" % name)
-    return t
+    raise ValueError("%s must be contiguous" % name)
 
 
 def _host(t, dtype, shape, name):
@@ -245,6 +249,8 @@ class Problem:
             raise MPBPError(s, "mpbp_create")
         self._h = h
         self.device = torch.cuda.current_device()
+        self._shapes = {"rho": (self.n1, self.n2), "u": (self.ncomp, self.n1, self.n2),
+                        "alpha": (self.npeaks,), "frames": (self.npeaks, self.nscan, self.m, self.m)}
 
     @classmethod
     def from_spec(cls, spec, scan):
@@ -269,15 +275,14 @@ class Problem:
 
     @property
     def shapes(self):
-        return {"rho": (self.n1, self.n2), "u": (self.ncomp, self.n1, self.n2),
-                "alpha": (self.npeaks,), "frames": (self.npeaks, self.nscan, self.m, self.m)}
+        return dict(self._shapes)
 
     def _check(self, s, what):
         if s != 0:
             raise MPBPError(s, "%s: %s" % (what, self._lib.mpbp_last_error(self._h).decode()))
 
     def _state(self, rho, u, alpha):
-        sh = self.shapes
+        sh = self._shapes
         _dev(rho, torch.float32, sh["rho"], "rho")
         _dev(u, torch.float32, sh["u"], "u")
         _dev(alpha, torch.float32, sh["alpha"], "alpha")
@@ -338,9 +343,9 @@ class Problem:
                     "mpbp_set_scan_offsets")
 
     def set_data(self, y, bg=None):
-        _dev(y, torch.float32, self.shapes["frames"], "y")
+        _dev(y, torch.float32, self._shapes["frames"], "y")
         if bg is not None:
-            _dev(bg, torch.float32, self.shapes["frames"], "bg")
+            _dev(bg, torch.float32, self._shapes["frames"], "bg")
         self._check(self._lib.mpbp_set_data(self._h, _p(y), _p(bg), _stream()), "mpbp_set_data")
 
     def object_build(self, rho, u, alpha, out=None):
@@ -354,7 +359,7 @@ class Problem:
     def forward(self, rho, u, alpha, out=None):
         self._state(rho, u, alpha)
         if out is None:
-            out = torch.empty(self.shapes["frames"], dtype=torch.float32, device=rho.device)
+            out = torch.empty(self._shapes["frames"], dtype=torch.float32, device=rho.device)
         self._check(self._lib.mpbp_forward(self._h, _p(rho), _p(u), _p(alpha), _p(out), _stream()),
                     "mpbp_forward")
         return out
@@ -365,8 +370,8 @@ class Problem:
         dev = rho.device
         if out is None:
             out = (torch.empty(1, dtype=torch.float64, device=dev),
-                   torch.empty(self.shapes["rho"], dtype=torch.float32, device=dev),
-                   torch.empty(self.shapes["u"], dtype=torch.float32, device=dev),
+                   torch.empty(self._shapes["rho"], dtype=torch.float32, device=dev),
+                   torch.empty(self._shapes["u"], dtype=torch.float32, device=dev),
                    torch.empty(self.npeaks, dtype=torch.float64, device=dev))
         loss, g_rho, g_u, g_alpha = out
         nfr = 0
@@ -407,7 +412,7 @@ class Problem:
     def loss_grad_phases(self, rho, phi, alpha, frames=None):
         """Per-peak-phase form: phi [D][n1][n2] in place of u; returns
         (loss [1] float64, g_rho, g_phi [D][n1][n2], g_alpha [D] float64)."""
-        sh = self.shapes
+        sh = self._shapes
         _dev(rho, torch.float32, sh["rho"], "rho")
         _dev(phi, torch.float32, (self.npeaks,) + tuple(sh["rho"]), "phi")
         _dev(alpha, torch.float32, sh["alpha"], "alpha")
@@ -424,16 +429,16 @@ class Problem:
 
     def illumination(self):
         """sum over frames of |P_m(r - s_j)|^2 on the object grid (mpbp_illumination)."""
-        out = torch.empty(self.shapes["rho"], dtype=torch.float32, device="cuda")
+        out = torch.empty(self._shapes["rho"], dtype=torch.float32, device="cuda")
         self._check(self._lib.mpbp_illumination(self._h, _p(out), _stream()), "mpbp_illumination")
         return out
 
     def unwrap_phases(self, wrapped, mask=None, out=None):
         """2-D unwrapping of D phase maps [D][n1][n2] (mpbp_unwrap_phases)."""
-        shp = (self.npeaks,) + tuple(self.shapes["rho"])
+        shp = (self.npeaks,) + tuple(self._shapes["rho"])
         _dev(wrapped, torch.float32, shp, "wrapped")
         if mask is not None:
-            _dev(mask, torch.float32, self.shapes["rho"], "mask")
+            _dev(mask, torch.float32, self._shapes["rho"], "mask")
         if out is None:
             out = torch.empty_like(wrapped)
         self._check(self._lib.mpbp_unwrap_phases(self._h, _p(wrapped), _p(mask), _p(out), _stream()),
@@ -442,9 +447,9 @@ class Problem:
 
     def project_displacement(self, u, mask=None):
         """Pi_U of Eq. 10 on u, in place (mpbp_project_displacement)."""
-        _dev(u, torch.float32, self.shapes["u"], "u")
+        _dev(u, torch.float32, self._shapes["u"], "u")
         if mask is not None:
-            _dev(mask, torch.float32, self.shapes["rho"], "mask")
+            _dev(mask, torch.float32, self._shapes["rho"], "mask")
         self._check(self._lib.mpbp_project_displacement(self._h, _p(u), _p(mask), _stream()),
                     "mpbp_project_displacement")
         return u
@@ -461,7 +466,7 @@ class Problem:
 
     def adam_step(self, frames, chi, u, alpha_t, state, mask=None):
         """One minibatch iteration of Alg. 1 on chi, u, alpha_t (updated in place)."""
-        sh = self.shapes
+        sh = self._shapes
         _dev(chi, torch.float32, sh["rho"], "chi")
         _dev(u, torch.float32, sh["u"], "u")
         _dev(alpha_t, torch.float32, sh["alpha"], "alpha_t")
@@ -473,7 +478,7 @@ class Problem:
 
     def adam_get_state(self):
         """(m_chi, v_chi, m_u, v_u, m_alpha, v_alpha) device copies of the moments."""
-        sh, dev = self.shapes, "cuda"
+        sh, dev = self._shapes, "cuda"
         out = (torch.empty(sh["rho"], device=dev), torch.empty(sh["rho"], device=dev),
                torch.empty(sh["u"], device=dev), torch.empty(sh["u"], device=dev),
                torch.empty(self.npeaks, dtype=torch.float64, device=dev),
@@ -495,7 +500,7 @@ class Problem:
     def loss_grad_host(self, rho, u, alpha, y=None, out=None):
         """Host-buffer variant (copies in, evaluates, copies out, synchronises).
         y: float32 counts, or uint16 photon counts (mpbp_loss_grad_host_counts16)."""
-        sh = self.shapes
+        sh = self._shapes
         _host(rho, torch.float32, sh["rho"], "rho")
         _host(u, torch.float32, sh["u"], "u")
         _host(alpha, torch.float32, sh["alpha"], "alpha")
