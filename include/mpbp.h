@@ -102,7 +102,9 @@ typedef struct {
   int32_t blocks_per_sm;   /* resident blocks per SM the schedule assumes      */
   int32_t num_sms;
   int32_t launches_loss_grad; /* kernels + memsets enqueued by mpbp_loss_grad  */
-  int32_t launches_step;      /* kernels + memsets enqueued by mpbp_step       */
+  int32_t launches_step;      /* kernels + memsets enqueued by mpbp_step
+                                 (both at most: the deterministic mode clears
+                                 its pieces only where frames leave gaps)     */
   int32_t precision;          /* MPBP_PRECISION_* of the gradient evaluations */
   int32_t tile_copies;        /* FFT kernels that take their inputs by TMA tile and
                                  bulk copies of unpadded rows: bit 0 the gradient

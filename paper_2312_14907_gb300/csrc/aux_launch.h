@@ -63,7 +63,6 @@ cudaError_t launch_loss_reduce(const double* part, long long n, double* loss, in
 // the deterministic gradient: acc [D][n1][n2] = per pixel, the fixed-order
 // sum of the plan's pieces covering it (pieces w columns wide; plan in
 // device memory)
-cudaError_t launch_det_reduce(const DetPlan* plan, cf* acc, int D, int n1, int n2, int w, int num_sms,
-                              cudaStream_t s);
+cudaError_t launch_det_reduce(const DetPlan* plan, cf* acc, int D, int n1, int n2, int w, cudaStream_t s);
 
 }  // namespace mpbp

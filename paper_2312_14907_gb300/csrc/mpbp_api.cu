@@ -147,6 +147,7 @@ struct mpbp_ctx {
   cf* det_pool = nullptr;
   size_t det_pool_elems = 0, det_pool_cap = 0;
   const DetPlan* det_plan = nullptr;
+  bool det_gaps = false;      // pieces with rows between their frames: cleared each time
   std::vector<void*> det_old;   // earlier plans' buffers a captured step may still use
   std::string last_error;
 };
@@ -233,6 +234,7 @@ mpbp_status det_prepare(mpbp_ctx* c, int grid) {
   const int W = c->M;
   const long long N = c->nframes;
   std::vector<DetPiece> pieces;
+  bool gaps = false;
   std::vector<int> b0(grid);
   for (int b = 0; b < grid; ++b) {
     const long long lo = N * b / grid, hi = N * (b + 1) / grid;
@@ -245,6 +247,8 @@ mpbp_status det_prepare(mpbp_ctx* c, int grid) {
         pieces.push_back(DetPiece{0, sp.x, sp.x, m, sp.y});   // rows: the last row start, for now
       } else {
         DetPiece& pc = pieces.back();
+        // rows that no frame reaches are never written back
+        if (sp.x > pc.rows + W) gaps = true;
         pc.row0 = std::min(pc.row0, sp.x);
         pc.rows = std::max(pc.rows, sp.x);
       }
@@ -256,16 +260,18 @@ mpbp_status det_prepare(mpbp_ctx* c, int grid) {
     pc.off = off;
     off += (long long)pc.rows * W;
   }
-  // per (peak, column, band of W rows): the pieces that reach into it, in
-  // piece order (a pixel's candidates; the sum takes those covering it)
-  const int nband = (c->n1 + W - 1) / W;
-  const long long nkey = (long long)c->D * c->n2 * nband;
+  // per (peak, tile of columns, band of W rows): the pieces that reach into
+  // it, in piece order (a pixel's candidates; the sum takes those covering it)
+  const int nband = (c->n1 + W - 1) / W, ntile = (c->n2 + kDetTile - 1) / kDetTile;
+  const long long nkey = (long long)c->D * ntile * nband;
   std::vector<int> cnt((size_t)nkey + 1, 0);
   auto each_key = [&](const DetPiece& pc, auto&& fn) {
     const int b0 = std::max(pc.row0, 0) / W, b1 = (std::min(pc.row0 + pc.rows, c->n1) - 1) / W;
     if (std::min(pc.row0 + pc.rows, c->n1) <= std::max(pc.row0, 0)) return;
-    for (int col = std::max(pc.y, 0); col < std::min(pc.y + W, c->n2); ++col)
-      for (int b = b0; b <= b1; ++b) fn(((long long)pc.mpk * c->n2 + col) * nband + b);
+    const int y0 = std::max(pc.y, 0), y1 = std::min(pc.y + W, c->n2);
+    if (y1 <= y0) return;
+    for (int t = y0 / kDetTile; t <= (y1 - 1) / kDetTile; ++t)
+      for (int b = b0; b <= b1; ++b) fn(((long long)pc.mpk * ntile + t) * nband + b);
   };
   for (const DetPiece& pc : pieces) each_key(pc, [&](long long k) { cnt[(size_t)k + 1]++; });
   for (long long i = 0; i < nkey; ++i) cnt[(size_t)i + 1] += cnt[(size_t)i];
@@ -322,6 +328,7 @@ mpbp_status det_prepare(mpbp_ctx* c, int grid) {
     return fail(c, MPBP_ERR_CUDA, "deterministic gradient: upload");
   c->det_plan = reinterpret_cast<const DetPlan*>(m + oD);
   c->det_grid = grid;
+  c->det_gaps = gaps;
   return MPBP_OK;
 }
 
@@ -344,13 +351,16 @@ cudaError_t launch_frames(const mpbp_ctx* c, const FrameArgs& fa, int grid, cuda
     f2.frames = c->strip_order;
   if (c->det) {
     f2.det = c->det_plan;
-    cudaError_t e = cudaMemsetAsync(c->det_pool, 0, sizeof(cf) * c->det_pool_elems, s);
+    // Every row of a piece is stored before it is read unless its frames
+    // leave gaps between them.
+    cudaError_t e = cudaSuccess;
+    if (c->det_gaps) e = cudaMemsetAsync(c->det_pool, 0, sizeof(cf) * c->det_pool_elems, s);
     if (e != cudaSuccess) return e;
     TmaMap tm = c->tm_grad;
     tm.tx_extra = c->test_tx_extra;
     e = frames_launch(c->M, f2, grid, false, s, &tm, c->fft_schedule);
     if (e != cudaSuccess) return e;
-    return launch_det_reduce(c->det_plan, c->acc, c->D, c->n1, c->n2, c->M, c->num_sms, s);
+    return launch_det_reduce(c->det_plan, c->acc, c->D, c->n1, c->n2, c->M, s);
   }
   if (!c->tile_grad || fa.O != c->O) return frames_launch(c->M, f2, grid, false, s, nullptr, c->fft_schedule);
   TmaMap tm = c->tm_grad;

@@ -88,9 +88,10 @@ struct DetPiece {
 };
 
 // The deterministic gradient's plan for one grid size: pieces in order,
-// each block's first piece, and per (peak, column, band of w rows) the
-// pieces reaching into it (CSR: col_start[D * n2 * bands + 1],
+// each block's first piece, and per (peak, tile of kDetTile columns, band of
+// w rows) the pieces reaching into it (CSR: col_start[D * tiles * bands + 1],
 // col_piece[...]) in piece order.
+constexpr int kDetTile = 32;
 struct DetPlan {
   cf* pool;
   const DetPiece* pieces;
