@@ -92,6 +92,11 @@ MPBP_DI void bulk_load_stream(uint32_t dst, const void* src, uint32_t bytes, uin
       : "memory");
 }
 
+// start moving `bytes` (a multiple of 16, from a 16-byte boundary) to L2
+MPBP_DI void bulk_prefetch(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // generic-proxy accesses of shared memory (ordered before this point by a
 // barrier) before the asynchronous copies that follow
 MPBP_DI void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
