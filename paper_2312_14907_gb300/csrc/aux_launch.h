@@ -4,6 +4,14 @@
 
 namespace mpbp {
 
+// the Adam moments in or out of the context: six copies in one launch
+struct MomentCopy {
+  uint32_t* dst[6];
+  const uint32_t* src[6];
+  long long words[6];
+};
+cudaError_t launch_moment_copy(const MomentCopy& a, int num_sms, cudaStream_t s);
+
 // illumination map: sum over frames of |P_m(r - s_j)|^2 (mpbp_alg1.cu)
 struct IllumArgs {
   const cf* probe;       // [Dp][M][M]

@@ -1,4 +1,5 @@
-// mpbp_alg1.cu -- the illumination map behind the final threshold of Alg. 1.
+// mpbp_alg1.cu -- beside Alg. 1's iteration: the illumination map behind its
+// final threshold, and the copies of the Adam moments for checkpoints.
 #include "aux_launch.h"
 
 namespace mpbp {
@@ -23,7 +24,31 @@ __global__ void illumination_kernel(IllumArgs a) {
   }
 }
 
+// blockIdx.y: which of the six arrays (a minibatch loop that resumes and saves
+// is bound by the host's launches: 12 copies of 2 us each became two launches)
+__global__ void moment_copy_kernel(const __grid_constant__ MomentCopy a) {
+  uint32_t* const d = a.dst[blockIdx.y];
+  const uint32_t* const q = a.src[blockIdx.y];
+  const long long n = a.words[blockIdx.y], stride = (long long)gridDim.x * blockDim.x;
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (((reinterpret_cast<uintptr_t>(d) | reinterpret_cast<uintptr_t>(q)) & 15) == 0) {
+    const long long n4 = n / 4;
+    for (long long k = i; k < n4; k += stride)
+      reinterpret_cast<uint4*>(d)[k] = reinterpret_cast<const uint4*>(q)[k];
+    i += 4 * n4;   // what is left
+  }
+  for (; i < n; i += stride) d[i] = q[i];
+}
+
 }  // namespace
+
+cudaError_t launch_moment_copy(const MomentCopy& a, int num_sms, cudaStream_t s) {
+  long long most = 1;
+  for (long long w : a.words) most = w > most ? w : most;
+  const long long b = (most + 1023) / 1024;
+  moment_copy_kernel<<<dim3((unsigned)(b < num_sms * 2 ? b : num_sms * 2), 6), 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_illumination(const IllumArgs& a, int num_sms, cudaStream_t s) {
   const long long n = (long long)a.nframes * a.m * a.m;

@@ -587,6 +587,33 @@ mpbp_status enqueue_loss_grad(mpbp_ctx* c, const float* rho, const float* u, con
   return MPBP_OK;
 }
 
+// The six moment arrays; theirs: the caller's side of the copies.  One launch
+// where that side is device memory, else (not a use the interface names) the
+// runtime's copies and what they answer.
+mpbp_status copy_moments(mpbp_ctx* c, void* const* to, const void* const* from, const void* const* theirs,
+                         cudaStream_t s) {
+  const long long np = c->npix, nu = c->npix * c->C;
+  const long long words[6] = {np, np, nu, nu, 2ll * c->D, 2ll * c->D};
+  MomentCopy a{};
+  bool device = true;
+  for (int i = 0; i < 6; ++i) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, theirs[i]) != cudaSuccess) cudaGetLastError();
+    device = device && at.type == cudaMemoryTypeDevice && at.device == c->device &&
+             (reinterpret_cast<uintptr_t>(theirs[i]) & 3) == 0;
+    a.dst[i] = static_cast<uint32_t*>(to[i]);
+    a.src[i] = static_cast<const uint32_t*>(from[i]);
+    a.words[i] = words[i];
+  }
+  if (device) {
+    MPBP_CUDA(c, launch_moment_copy(a, c->num_sms, s));
+    return MPBP_OK;
+  }
+  for (int i = 0; i < 6; ++i)
+    MPBP_CUDA(c, cudaMemcpyAsync(to[i], from[i], sizeof(uint32_t) * words[i], cudaMemcpyDeviceToDevice, s));
+  return MPBP_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1400,15 +1427,9 @@ mpbp_status mpbp_adam_get_state(mpbp_ctx* c, float* m_chi, float* v_chi, float* 
   if (!c || !m_chi || !v_chi || !m_u || !v_u || !m_alpha || !v_alpha)
     return fail(c, MPBP_ERR_INVALID_ARG, "null argument");
   if (!c->adam_buf) return fail(c, MPBP_ERR_NO_DATA, "mpbp_adam_init first");
-  cudaStream_t s = S(stream);
-  const long long np = c->npix, nu = c->npix * c->C;
-  MPBP_CUDA(c, cudaMemcpyAsync(m_chi, c->m_chi, sizeof(float) * np, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(v_chi, c->v_chi, sizeof(float) * np, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(m_u, c->m_u, sizeof(float) * nu, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(v_u, c->v_u, sizeof(float) * nu, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(m_alpha, c->m_a, sizeof(double) * c->D, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(v_alpha, c->v_a, sizeof(double) * c->D, cudaMemcpyDeviceToDevice, s));
-  return MPBP_OK;
+  void* const to[6] = {m_chi, v_chi, m_u, v_u, m_alpha, v_alpha};
+  const void* const from[6] = {c->m_chi, c->v_chi, c->m_u, c->v_u, c->m_a, c->v_a};
+  return copy_moments(c, to, from, to, S(stream));
 }
 
 mpbp_status mpbp_adam_set_state(mpbp_ctx* c, const float* m_chi, const float* v_chi, const float* m_u,
@@ -1417,15 +1438,9 @@ mpbp_status mpbp_adam_set_state(mpbp_ctx* c, const float* m_chi, const float* v_
   if (!c || !m_chi || !v_chi || !m_u || !v_u || !m_alpha || !v_alpha)
     return fail(c, MPBP_ERR_INVALID_ARG, "null argument");
   if (!c->adam_buf) return fail(c, MPBP_ERR_NO_DATA, "mpbp_adam_init first");
-  cudaStream_t s = S(stream);
-  const long long np = c->npix, nu = c->npix * c->C;
-  MPBP_CUDA(c, cudaMemcpyAsync(c->m_chi, m_chi, sizeof(float) * np, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(c->v_chi, v_chi, sizeof(float) * np, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(c->m_u, m_u, sizeof(float) * nu, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(c->v_u, v_u, sizeof(float) * nu, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(c->m_a, m_alpha, sizeof(double) * c->D, cudaMemcpyDeviceToDevice, s));
-  MPBP_CUDA(c, cudaMemcpyAsync(c->v_a, v_alpha, sizeof(double) * c->D, cudaMemcpyDeviceToDevice, s));
-  return MPBP_OK;
+  void* const to[6] = {c->m_chi, c->v_chi, c->m_u, c->v_u, c->m_a, c->v_a};
+  const void* const from[6] = {m_chi, v_chi, m_u, v_u, m_alpha, v_alpha};
+  return copy_moments(c, to, from, from, S(stream));
 }
 
 mpbp_status mpbp_loss_grad_phases(mpbp_ctx* c, const float* rho, const float* phi, const float* alpha,

@@ -47,6 +47,27 @@ enum ObjectForm {
              // block 0 also counts the Adam step
 };
 
+// one pixel's inputs of the object synthesis
+struct ObjIn {
+  float r, mask;
+  float uc[kMaxComp];
+};
+
+template <int FORM>
+__device__ __forceinline__ ObjIn object_load(const ObjectArgs& a, long long p) {
+  ObjIn in;
+  in.mask = 1.0f;
+  if constexpr (FORM == kObjAdam) {
+    in.r = a.ad.chi[p];
+    if (a.ad.mask) in.mask = a.ad.mask[p];
+  } else {
+    in.r = a.rho[p];
+  }
+#pragma unroll
+  for (int c = 0; c < kMaxComp; ++c) in.uc[c] = FORM != kObjPhi && c < a.C ? a.u[c * a.npix + p] : 0.f;
+  return in;
+}
+
 // block bid of the nblk that work on a
 template <int FORM>
 __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int nblk) {
@@ -54,6 +75,10 @@ __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int n
   const int pad = a.pitch - a.n2;
   const long long ostride = a.npix / a.n2 * a.pitch;
   __shared__ float s_alpha[kMaxPeaks];
+  // the first pixel's reads are in flight beside the peaks'
+  long long p = (long long)bid * blockDim.x + threadIdx.x;
+  ObjIn in{};
+  if (p < a.npix) in = object_load<FORM>(a, p);
   if (threadIdx.x < a.D) {
     const int m = threadIdx.x;
     if constexpr (FORM == kObjAdam) s_alpha[m] = m == 0 ? 1.0f : expf(a.ad.alpha_t[m]);
@@ -70,14 +95,9 @@ __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int n
     if (threadIdx.x == 32) st->bc2 = one_minus_pow(st->beta2, t);
   }
   __syncthreads();
-  for (long long p = (long long)bid * blockDim.x + threadIdx.x; p < a.npix; p += stride) {
+  while (p < a.npix) {
     const long long q = pad ? p + (unsigned)p / (unsigned)a.n2 * (long long)pad : p;   // npix < 2^31
-    float r;
-    if constexpr (FORM == kObjAdam) r = (a.ad.mask ? a.ad.mask[p] : 1.0f) * expf(a.ad.chi[p]);
-    else r = a.rho[p];
-    float uc[kMaxComp];
-#pragma unroll
-    for (int c = 0; c < kMaxComp; ++c) uc[c] = FORM != kObjPhi && c < a.C ? a.u[c * a.npix + p] : 0.f;
+    const float r = FORM == kObjAdam ? in.mask * expf(in.r) : in.r;
 #pragma unroll
     for (int m = 0; m < kMaxPeaks; ++m) {
       if (m < a.D) {
@@ -87,13 +107,15 @@ __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int n
         } else {
           float arg = 0.f;
 #pragma unroll
-          for (int c = 0; c < kMaxComp; ++c) arg = fmaf(a.pc.kpi[m][c], uc[c], arg);
+          for (int c = 0; c < kMaxComp; ++c) arg = fmaf(a.pc.kpi[m][c], in.uc[c], arg);
           sincospif(arg, &sn, &cs);   // exp(i phi), phi = pi * arg
         }
         const float amp = s_alpha[m] * r;
         reinterpret_cast<float2*>(a.O)[m * ostride + q] = make_float2(amp * cs, amp * sn);
       }
     }
+    p += stride;
+    if (p < a.npix) in = object_load<FORM>(a, p);
   }
 }
 
