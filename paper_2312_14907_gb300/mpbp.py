@@ -216,7 +216,9 @@ def _dev(t, dtype, shape, name):
         raise TypeError("%s must be %s, got %s" % (name, dtype, t.dtype))
     if tuple(t.shape) != tuple(shape):
         raise ValueError("%s must have shape %s, got %s" % (name, tuple(shape), tuple(t.shape)))
-    raise ValueError("%s must be contiguous" % name)
+    if not t.is_contiguous():
+        raise ValueError("%s must be contiguous" % name)
+    return t
 
 
 def _host(t, dtype, shape, name):
