@@ -130,6 +130,7 @@ struct mpbp_ctx {
   // phase unwrapping / projector workspace (lazily allocated)
   void* uw_buf = nullptr;
   UnwrapArgs uw{};
+  bool uw_lists_dirty = true;   // the closing kernel clears the tiles' list counts; not yet, or its launch failed
   float *pj_phi = nullptr, *pj_wrapped = nullptr;
   int uw_grid = 0;
   // one optimizer step captured as a CUDA graph (mpbp_step_capture)
@@ -1473,10 +1474,6 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
     return fail(c, MPBP_ERR_OOM, "unwrap workspace");
   }
   char* p = static_cast<char*>(b);
-  if (cudaMemset(p + o_l, 0, sizeof(int) * (5 * c->D + 1)) != cudaSuccess) {
-    cudaFree(b);
-    return fail(c, MPBP_ERR_CUDA, "unwrap workspace");
-  }
   c->uw_buf = b;
   UnwrapArgs& a = c->uw;
   a.rel = reinterpret_cast<float*>(p + o_rel);
@@ -1520,6 +1517,9 @@ UnwrapArgs unwrap_args(const mpbp_ctx* c, const float* wrapped, const float* mas
 
 mpbp_status enqueue_unwrap(mpbp_ctx* c, const UnwrapArgs& a, cudaStream_t s) {
   if (unwrap_by_tiles(a)) {
+    if (c->uw_lists_dirty)
+      MPBP_CUDA(c, cudaMemsetAsync(a.lists, 0, sizeof(int) * 2 * c->D, s));
+    c->uw_lists_dirty = true;
     MPBP_CUDA(c, unwrap_tiles_launch(a, c->uw_grid, s));
     return MPBP_OK;
   }
@@ -1575,7 +1575,10 @@ mpbp_status mpbp_unwrap_phases(mpbp_ctx* c, const float* wrapped, const float* m
   const UnwrapArgs a = unwrap_args(c, wrapped, mask, out);
   r = enqueue_unwrap(c, a, s);
   if (r != MPBP_OK) return r;
-  if (unwrap_by_tiles(a)) MPBP_CUDA(c, unwrap_close_launch(a, c->num_sms, s));
+  if (unwrap_by_tiles(a)) {
+    MPBP_CUDA(c, unwrap_close_launch(a, c->num_sms, s));
+    c->uw_lists_dirty = false;
+  }
   return MPBP_OK;
 }
 
@@ -1605,6 +1608,7 @@ mpbp_status mpbp_project_displacement(mpbp_ctx* c, float* u, const float* mask, 
   r = enqueue_unwrap(c, a, s);
   if (r != MPBP_OK) return r;
   MPBP_CUDA(c, project_correct_launch(pa, a, unwrap_by_tiles(a), c->num_sms, s));
+  if (unwrap_by_tiles(a)) c->uw_lists_dirty = false;
   return MPBP_OK;
 }
 
