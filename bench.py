@@ -849,7 +849,7 @@ def alg1_block(torch, prob, spec, x, flush, stream):
         "iteration": "Alg. 1 minus the projector: minibatch of %d frames, Adam (0.01 u, 0.1 chi, 0.1 alpha)" % bsz,
         "ms_per_epoch": ep_ms, "minibatches_per_epoch": len(batches[0]),
         "ms_per_minibatch": ep_ms / len(batches[0]), "value": spec.nframes / (ep_ms / 1e3), "unit": UNIT,
-        "launches_per_minibatch": 5,
+        "launches_per_minibatch": 3,
         "graph": {"ms_per_epoch": gep_ms, "ms_per_minibatch": gep_ms / len(batches[0]),
                   "value": spec.nframes / (gep_ms / 1e3), "unit": UNIT,
                   "note": "each epoch one CUDA graph replay (minibatch slices of a fixed order buffer)"},
