@@ -2,7 +2,7 @@
 none reaches (its pieces are then cleared on every call), where they just touch,
 and where pieces lie beside, across and off the grid's edges: against the FP64
 oracle (the parity tests' tolerances) and bit for bit on repetition, on a grid
-whose sides are no multiples of the 32 x 32 pixels a block sums."""
+whose sides are no multiples of the 8 x 32 pixels a block sums."""
 import numpy as np
 import pytest
 import torch
