@@ -4,6 +4,7 @@
 //   A6/A7 tail: gradient assembly from the patch accumulator
 //   A8  fixed-order FP64 reductions, the line-search decision and the update
 //       of mpbp_step (applied by the gradient assembly, pixel by pixel)
+#include "adam_bias.h"
 #include "aux_launch.h"
 
 #include <algorithm>
@@ -13,31 +14,6 @@ namespace mpbp {
 // ----------------------------------------------------------------------------
 // A1: objects
 // ----------------------------------------------------------------------------
-// 1 - b^t for 0 <= b < 1, t >= 1: binary powers, each kept as an FP64 pair
-// (hi + lo), so that the result is good to an ulp or two for every t; the
-// loop is far shorter than the library's pow, whose latency one thread would
-// put in front of the whole step (minibatch step 47 -> 26 us with the
-// fusions below, see the Adam form of the object synthesis).
-__device__ double one_minus_pow(double b, long long t) {
-  struct Dd {
-    double h, l;
-  };
-  auto mul = [](Dd x, Dd y) {
-    const double p = x.h * y.h;
-    const double e = fma(x.h, y.h, -p) + fma(x.h, y.l, x.l * y.h);
-    const double h = p + e;
-    return Dd{h, e - (h - p)};
-  };
-  Dd r{1.0, 0.0}, x{b, 0.0};
-  while (true) {
-    if (t & 1) r = mul(r, x);
-    t >>= 1;
-    if (t == 0) break;
-    x = mul(x, x);
-  }
-  return (1.0 - r.h) - r.l;
-}
-
 // Where the phases and amplitudes of O come from.
 enum ObjectForm {
   kObjU,     // rho, alpha; phases from u
@@ -86,7 +62,7 @@ __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int n
   }
   if (FORM == kObjAdam && bid == 0) {
     mpbp_adam_state* st = a.ad.st;
-    const long long t = st->t + 1;
+    const long long t = (long long)((unsigned long long)st->t + 1ull);   // any stored count
     __syncthreads();   // every thread has read the old count
     if (threadIdx.x == 0) {
       st->t = t;
