@@ -101,22 +101,25 @@ MPBP_DI void bulk_prefetch(const void* src, uint32_t bytes) {
 // barrier) before the asynchronous copies that follow
 MPBP_DI void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// One thread: wait (at most kBulkWaitNs) for the phase with the given
-// parity; false if the copies did not land.
-MPBP_DI bool bulk_wait_thread(uint32_t bar, uint32_t parity) {
+// Every thread of the warp: wait (at most kBulkWaitNs) for the phase with the
+// given parity; false in the threads that did not see the copies land.  The
+// warp is converged behind it, which the tensor-memory instructions that
+// follow require: its lanes may leave the loop in different passes.
+MPBP_DI bool bulk_wait_warp(uint32_t bar, uint32_t parity) {
   uint32_t done = mbar_test(bar, parity);
   if (!done) {
     const unsigned long long t0 = timer_ns();
     while (!(done = mbar_test(bar, parity)) && timer_ns() - t0 < kBulkWaitNs) {
     }
   }
+  __syncwarp();
   return done != 0;
 }
 
 // Every thread of the block: wait (at most kBulkWaitNs) for the phase with
 // the given parity; block-uniform result, false if the copies did not land.
 MPBP_DI bool bulk_wait(uint32_t bar, uint32_t parity) {
-  return __syncthreads_and((int)bulk_wait_thread(bar, parity)) != 0;
+  return __syncthreads_and((int)bulk_wait_warp(bar, parity)) != 0;
 }
 
 // a block's input copies: its mbarrier and the phase it waits for next

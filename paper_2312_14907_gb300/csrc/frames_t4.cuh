@@ -133,6 +133,7 @@ MPBP_DI void t4_fetch(const FrameArgs& p, const T4Group<M>& g, const FrameRef& r
         for (int b = 0; b < M / C::AB; ++b) bulk_load_stream(dst + b * C::ABAND, src + b * C::AB * M, kBand, bs.bar);
       }
     }
+    __syncwarp();
   } else {
     const PatchSrc q = patch_src<M>(p, r);
     // a rolled loop keeps the copies' addresses out of the registers the

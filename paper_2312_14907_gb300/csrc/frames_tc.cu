@@ -151,11 +151,16 @@ MPBP_DI void pair_columns(const float (&d)[64], int po, float (&re)[32], float (
 
 MPBP_DI float abs_max(float m, float x) { return fmaxf(m, fabsf(x)); }
 
-MPBP_DI void group_bar(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(GT) : "memory"); }
+// (bar.sync and bar.red are warp-wide, as the tensor-memory instructions are)
+MPBP_DI void group_bar(int id) {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(GT) : "memory");
+}
 
 // group barrier that also returns whether v != 0 in every thread of the group
 MPBP_DI int group_bar_and(int id, int v) {
   int r;
+  __syncwarp();
   asm volatile(
       "{\n.reg .pred q, a;\nsetp.ne.s32 q, %1, 0;\nbar.red.and.pred a, %2, %3, q;\nselp.s32 %0, 1, 0, a;\n}"
       : "=r"(r)
@@ -327,6 +332,7 @@ MPBP_DI void tc_wait(TcGroup& G, int* err) {
   G.phase ^= 1u;
   const int ok = group_bar_and(G.id, G.ok && done);
   if (G.ok && !ok && G.t == 0) atomicOr(err, kErrTimeout);
+  __syncwarp();
   G.ok = ok;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
@@ -369,6 +375,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (blockIdx.x == 0 && tid == 0 && p.arrivals) *p.arrivals = 0u;
 
   if (tid < 32) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&taddr_holder)),
                  "r"(TMEM_COLS)
                  : "memory");
@@ -600,6 +607,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     w128[tid] = cf{cs, -sn};
   }
   if (tid < 32) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&taddr_holder)),
                  "r"(TMEM_COLS)
                  : "memory");

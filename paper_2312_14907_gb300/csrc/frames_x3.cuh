@@ -229,6 +229,7 @@ MPBP_DI void x3_fetch_amp_tma(const FrameArgs& p, const X3Roles& r, const FrameR
     mbar_arrive_tx(bs.bar, (fr.valid ? kPatch + kAmp : 0u) + tm->tx_extra);
     if (fr.valid) bulk_load_stream(smem_addr(abuf), p.aT + (long long)fr.f * M * M, kAmp, bs.bar);
   }
+  __syncwarp();
 }
 
 MPBP_DI void x3_fetch_patch_tma(const X3Roles& r, const FrameRef& fr, cf* buf, const BulkState& bs,
@@ -237,6 +238,7 @@ MPBP_DI void x3_fetch_patch_tma(const X3Roles& r, const FrameRef& fr, cf* buf, c
     fence_async_smem();
     tile_load_3d(smem_addr(buf), &tm->map, fr.s.y - (fr.s.y & 1), fr.s.x, fr.mpk, bs.bar);
   }
+  __syncwarp();
 }
 
 // inputs of frame fr: the patch tile and, but for the forward model, sqrt(y)
@@ -259,6 +261,7 @@ MPBP_DI void x3_fetch(const FrameArgs& p, const X3Roles& r, const FrameRef& fr, 
         if constexpr (!FWD) bulk_load_stream(smem_addr(abuf), p.aT + (long long)fr.f * M * M, kAmp, bs.bar);
       }
     }
+    __syncwarp();
   } else {
     const PatchSrc q = patch_src<M>(p, fr);
 #pragma unroll 2
@@ -292,7 +295,7 @@ MPBP_DI void x3_frame(const FrameArgs& p, const X3Roles& r, const FrameRef& cur,
   tmem_ld16(tp, w[0]);
   bool ok = true;
   if constexpr (TMA) {
-    ok = bulk_wait_thread(bs.bar, bs.parity);   // the block agrees on it below
+    ok = bulk_wait_warp(bs.bar, bs.parity);   // the block agrees on it below
     bs.parity ^= 1u;
   } else {
     cp_async_wait_all();
@@ -649,6 +652,7 @@ MPBP_DI double x3_run(const FrameArgs& p, const TmaMap* tm, int lo, int hi, X3Bl
       // transformed (512^2, 5,043 shifted probes: 494 -> 454 us a call)
       if (p.probe_stride < 0 && threadIdx.x == 0 && nxt.valid)
         bulk_prefetch(frame_probe(p, nxt, M * M), M * M * (uint32_t)sizeof(cf));
+      __syncwarp();
     }
     x3_frame<TMA, LOSS, BG, DET, FWD>(p, b.r, cur, nxt, [&](float fl) { lsum += (double)fl; }, b.bs, tm, b.buf, b.abuf,
                                       b.tp, b.ta, tab, win);

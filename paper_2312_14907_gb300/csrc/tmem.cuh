@@ -3,6 +3,11 @@
 // lane (the 32x32b shape: thread i of a warp reaches lane 32 (warp mod 4) + i
 // of the SM's 128 lanes), and the waits and fences that order them.
 //
+// These instructions are warp-wide (.sync.aligned): the warp has to be
+// converged.  So a branch that some of its lanes take ahead of them (one
+// thread issuing copies, a wait that lanes leave in different passes, a
+// guarded store) ends with __syncwarp().
+//
 // A warp may only touch the lane quarter of its index modulo 4, so the warps
 // w, w + 4, w + 8, ... share lanes and are given disjoint column ranges.
 #pragma once
@@ -17,6 +22,7 @@ namespace mpbp {
 // address to the shared-memory word at smem_dst; then give up the right to
 // allocate more, so that other blocks on the SM are not kept waiting
 MPBP_DI void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols)
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
