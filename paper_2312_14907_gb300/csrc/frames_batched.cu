@@ -134,7 +134,10 @@ __global__ void __launch_bounds__(T2Cfg<M>::T, T2Cfg<M>::MINB) frames_batched_m(
         },
         &bs, TMA ? &b.tmaps[item.x] : nullptr);
     if (TMA && !bs.ok) {
-      if (threadIdx.x == 0) atomicOr(sp[cs].err, kErrTimeout);
+      // this frame's problem and every problem whose later frames the block leaves out
+      const long long step = (long long)gridDim.x * blockDim.x;
+      for (long long j = it + (long long)gridDim.x * threadIdx.x; j < b.nitems; j += step)
+        atomicOr(b.probs[b.items[j].x].err, kErrTimeout);
       break;
     }
     cs = ns;

@@ -45,6 +45,9 @@ __global__ void __launch_bounds__(X3Cfg::T, 1) frames_x3_batch(const __grid_cons
       const double lsum = sp.bgT ? x3_run<true, false, true, false, false>(sp, a.tmaps + k, l, h, b, tab)
                                  : x3_run<true, false, false, false, false>(sp, a.tmaps + k, l, h, b, tab);
       tot = block_sum_d<X3Cfg::T>(lsum, red);   // barriers: sp may be overwritten
+    } else if (l < h && threadIdx.x == 0) {
+      // a wait ran out in an earlier problem: this one misses the block's frames too
+      atomicOr(a.probs[k].err, kErrTimeout);
     }
     // every (problem, block) slot is written, so none needs clearing
     if (threadIdx.x == 0) a.frame_part[(long long)k * gridDim.x + blockIdx.x] = tot;
