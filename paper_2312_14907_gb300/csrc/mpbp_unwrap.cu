@@ -385,7 +385,9 @@ __global__ void __launch_bounds__(kUnwrapThreads) unwrap_tile_kernel(UnwrapArgs 
 constexpr int kMapThreads = 1024;
 constexpr int kMapEdges = 8;
 
+// (warp-wide instructions: the lanes come out of strided loops of their own)
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 

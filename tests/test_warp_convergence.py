@@ -1,5 +1,5 @@
 """The warp-wide instructions of tensor memory (tcgen05 .sync.aligned) and of
-the named barriers (bar.sync, bar.red) need a converged warp.  Read off the
+the named and cluster barriers (bar.sync, bar.red, barrier.cluster) need a converged warp.  Read off the
 sources: each place where lanes of a warp part ways ahead of one -- the bounded
 wait on a copy, the branch in which one thread issues copies, the allocation
 behind a thread's own work -- ends in __syncwarp().  (Text only: a kernel that
@@ -65,12 +65,13 @@ def test_allocation_starts_converged(name):
         assert s[:a].rstrip().endswith("__syncwarp();")
 
 
-def test_named_barriers_start_converged():
-    s = _text("frames_tc.cu")
-    for f in ("group_bar", "group_bar_and"):
-        i, j = _block(s, s.index(f + "(int id"))
-        body = s[i:j]
-        assert "__syncwarp();" in body[:body.index("asm volatile")]
+@pytest.mark.parametrize("name,fn", [("frames_tc.cu", "group_bar(int"), ("frames_tc.cu", "group_bar_and("),
+                                     ("frames.cuh", "void sync()"), ("mpbp_unwrap.cu", "void cluster_sync(")])
+def test_named_and_cluster_barriers_start_converged(name, fn):
+    s = _text(name)
+    i, j = _block(s, s.index(fn))
+    body = s[i:j]
+    assert "__syncwarp();" in body[:body.index("asm volatile")]
 
 
 def test_no_guarded_store_ahead_of_tensor_memory():
@@ -86,6 +87,7 @@ def test_no_guarded_store_ahead_of_tensor_memory():
         assert "red_add_v2(" not in s[a:b]
 
 
-def test_every_source_with_tensor_memory_is_known():
-    names = {os.path.basename(f) for f in glob.glob(os.path.join(CSRC, "*")) if "sync.aligned" in open(f).read()}
-    assert names == {"tmem.cuh", "frames_tc.cu"}
+def test_every_source_with_warp_wide_instructions_is_known():
+    wide = re.compile(r"sync\.aligned|barrier\.cluster|bar\.sync|bar\.red")
+    names = {os.path.basename(f) for f in glob.glob(os.path.join(CSRC, "*")) if wide.search(_text(os.path.basename(f)))}
+    assert names == {"tmem.cuh", "frames_tc.cu", "frames.cuh", "mpbp_unwrap.cu"}
