@@ -1460,12 +1460,21 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
   if (c->uw_buf) return MPBP_OK;
   if (!unwrap_prepare(c->num_sms, &c->uw_grid)) return fail(c, MPBP_ERR_CUDA, "unwrap kernel cannot run here");
   const long long nodes = c->npix * c->D;
+  UnwrapArgs& a = c->uw;
+  a.n1 = c->n1;
+  a.n2 = c->n2;
+  a.max_blocks = unwrap_map_blocks();
+  if (unwrap_by_tiles(a)) {
+    a.comp_cap = unwrap_comp_cap(c->n1, c->n2);
+    a.spill_cap = unwrap_spill_cap(c->n1, c->n2);
+  }
   Carver cv;
   const size_t o_rel = cv.take<float>(nodes), o_p = cv.take<int>(nodes), o_o = cv.take<int>(nodes),
                o_p2 = cv.take<int>(nodes), o_o2 = cv.take<int>(nodes), o_hp = cv.take<int>(nodes),
                o_ho = cv.take<int>(nodes), o_mn = cv.take<int>(nodes),
                o_b = cv.take<unsigned long long>(nodes), o_ek = cv.take<unsigned long long>(2 * nodes),
-               o_f = cv.take<int>(3), o_bc = cv.take<unsigned>(2), o_l = cv.take<int>(5 * c->D + 1),
+               o_f = cv.take<int>(3), o_bc = cv.take<unsigned>(2), o_l = cv.take<int>(5 * c->D),
+               o_cp = cv.take<int>(6 * c->D * a.comp_cap), o_ee = cv.take<int2>(c->D * a.spill_cap),
                o_phi = cv.take<float>(nodes), o_w = cv.take<float>(nodes);
   void* b = nullptr;
   MPBP_CUDA(c, cudaStreamSynchronize(s));
@@ -1475,7 +1484,6 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
   }
   char* p = static_cast<char*>(b);
   c->uw_buf = b;
-  UnwrapArgs& a = c->uw;
   a.rel = reinterpret_cast<float*>(p + o_rel);
   a.parent = reinterpret_cast<int*>(p + o_p);
   a.off = reinterpret_cast<int*>(p + o_o);
@@ -1491,16 +1499,14 @@ mpbp_status unwrap_setup(mpbp_ctx* c, cudaStream_t s) {
   a.bar_gen = a.bar_count + 1;
   a.lists = reinterpret_cast<int*>(p + o_l);
   a.map_flags = a.lists + 2 * c->D;
-  a.need_global = a.map_flags + 3 * c->D;
+  a.comps = reinterpret_cast<int*>(p + o_cp);
+  a.edge_ends = reinterpret_cast<int2*>(p + o_ee);
   a.err = c->err;
   a.npix = c->npix;
   a.nodes = nodes;
-  a.n1 = c->n1;
-  a.n2 = c->n2;
   int rounds = 2;
   while ((1ll << rounds) < nodes) ++rounds;
   a.max_rounds = rounds + 2;
-  a.max_blocks = unwrap_map_blocks();
   c->pj_phi = reinterpret_cast<float*>(p + o_phi);
   c->pj_wrapped = reinterpret_cast<float*>(p + o_w);
   return MPBP_OK;
@@ -1520,12 +1526,12 @@ mpbp_status enqueue_unwrap(mpbp_ctx* c, const UnwrapArgs& a, cudaStream_t s) {
     if (c->uw_lists_dirty)
       MPBP_CUDA(c, cudaMemsetAsync(a.lists, 0, sizeof(int) * 2 * c->D, s));
     c->uw_lists_dirty = true;
-    MPBP_CUDA(c, unwrap_tiles_launch(a, c->uw_grid, s));
+    MPBP_CUDA(c, unwrap_tiles_launch(a, s));
     return MPBP_OK;
   }
   MPBP_CUDA(c, cudaMemsetAsync(a.flags, 0, sizeof(int) * 3, s));
   MPBP_CUDA(c, cudaMemsetAsync(a.bar_count, 0, sizeof(unsigned) * 2, s));
-  MPBP_CUDA(c, unwrap_launch(a, c->uw_grid, false, s));
+  MPBP_CUDA(c, unwrap_launch(a, c->uw_grid, s));
   return MPBP_OK;
 }
 

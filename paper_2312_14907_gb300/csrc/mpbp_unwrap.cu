@@ -25,14 +25,14 @@
 //   - maps of at most 1,280 tiles (572^2 pixels): one kernel contracts the
 //     16 x 16 tiles (reliabilities and edge keys formed on the way) and lists
 //     the components and edges that are left; one cluster of 8 or 16 blocks
-//     per map runs the remaining rounds on those lists; the caller's closing
-//     kernel applies the offsets.  What bounds it is the chain of rounds (three
-//     256^2 maps: 119 us a projector call, against 237);
-//   - larger maps, and maps whose lists do not fit that cluster: one
-//     cooperative launch (every block resident), bound by its grid barriers
-//     (~5 us each, about 35 of them; three 256^2 maps: 226 us), which are
-//     bounded in time: if one runs out, the block records kErrTimeout and
-//     leaves, and the rest run out at their next barrier.
+//     per map runs the remaining rounds on those lists, which hold whatever a
+//     map of such a size leaves; the caller's closing kernel applies the
+//     offsets.  What bounds it is the chain of rounds (three 256^2 maps: 120 us
+//     a projector call, against 237);
+//   - larger maps: one cooperative launch (every block resident), bound by its
+//     grid barriers (~5 us each, about 35 of them; three 256^2 maps: 226 us),
+//     which are bounded in time: if one runs out, the block records
+//     kErrTimeout and leaves, and the rest run out at their next barrier.
 #include <cmath>
 #include <climits>
 
@@ -283,14 +283,20 @@ __device__ void local_contract(const UnwrapArgs& a) {
 //   off2[root]        what is added to off for the output
 //   of component l of a map (at the map's first node + l): hook_off its root,
 //   minnode its lowest node, hook_parent that node's off
-//   ekey              per map, npix / 2 listed edges' keys, then npix / 2
-//                     places each for the components' parent and offset (two
-//                     buffers), hook and hook offset
+//   ekey              per map, the listed edges' keys (a grid has fewer than
+//                     2 npix edges)
 //   best              of component l of a map, as everywhere
+//   comps             per map, comp_cap places each for the components' parent
+//                     and offset (two buffers), hook and hook offset
+//   edge_ends         per map, the components at the ends of listed edge
+//                     kMapRegEdges + k
 //   lists[2 m]        components and edges listed (zero between calls)
+// How many a map leaves: a listed component holds a pixel with an edge out of
+// its tile, so at most 60 a tile; counted on whole 512^2 grids, 16 (smooth
+// phases) to 21 (random) components and 217 (smooth), 139 (noisy), 145
+// (random) edges a tile, about half as many inside a disc of half the area.
 // ----------------------------------------------------------------------------
 
-__device__ __forceinline__ int map_cap(const UnwrapArgs& a) { return (int)(a.npix / 2); }   // components, edges
 __device__ __forceinline__ unsigned long long* map_keys(const UnwrapArgs& a, int m) { return a.ekey + 2 * m * a.npix; }
 
 // one block per tile: reliabilities, edge keys, contraction, lists
@@ -306,11 +312,6 @@ __global__ void __launch_bounds__(kUnwrapThreads) unwrap_tile_kernel(UnwrapArgs 
   const int m = blockIdx.x / (tpr * tpc), rem = blockIdx.x - m * (tpr * tpc);
   const int i0 = rem / tpr * kTile, j0 = rem % tpr * kTile;
   const long long base = (long long)m * a.npix;
-  if (blockIdx.x == 0 && t < 6) {   // for the cooperative kernel that may follow
-    if (t < 3) a.flags[t] = 0;
-    else if (t < 5) a.bar_count[t - 3] = 0u;
-    else *a.need_global = 0;
-  }
   for (int k = t; k < W * W; k += kUnwrapThreads) {
     const int i = i0 - 2 + k / W, j = j0 - 2 + k % W;
     const bool ok = i >= 0 && j >= 0 && i < n1 && j < n2 && in_mask(a, (long long)i * n2 + j);
@@ -374,16 +375,18 @@ __global__ void __launch_bounds__(kUnwrapThreads) unwrap_tile_kernel(UnwrapArgs 
         a.off2[v] = -s.lo[lm];
       }
     }
-    const int k = s_at[1] + le, cap = map_cap(a);   // past it, the map kernel gives the work up
+    const long long k = s_at[1] + le;
     unsigned long long* const ek = map_keys(a, m);
-    if (er && k < cap) ek[k] = kr;
-    if (ed && k + er < cap) ek[k + er] = kd;
+    if (er && k < 2 * a.npix) ek[k] = kr;   // (always, from counts that start at 0)
+    if (ed && k + er < 2 * a.npix) ek[k + er] = kd;
   }
 }
 
-// A map's cluster: threads a block, edges a thread keeps in registers.
+// A map's cluster: threads a block, edges a thread keeps in registers (the
+// smallest cluster's are the ones that need no place in edge_ends).
 constexpr int kMapThreads = 1024;
 constexpr int kMapEdges = 8;
+constexpr int kMapRegEdges = 8 * kMapThreads * kMapEdges;
 
 // (warp-wide instructions: the lanes come out of strided loops of their own)
 __device__ __forceinline__ void cluster_sync() {
@@ -396,23 +399,24 @@ __device__ __forceinline__ void cluster_sync() {
 // the reads around it, against 5 us for the grid's; one block instead of
 // eight, its state in shared memory, took longer than the whole grid: it is
 // bound by its SM's issue and by one lane a clock for its scattered reads).
+// A thread takes every all-th listed edge: the first kMapEdges in registers,
+// the rest in L2, where each round leaves those between two components at the
+// front of the thread's own places.
 __global__ void __launch_bounds__(kMapThreads) unwrap_map_kernel(UnwrapArgs a, int blocks) {
   const int m = blockIdx.x / blocks;
   const int t = (blockIdx.x % blocks) * kMapThreads + threadIdx.x;   // within the cluster
   const int all = blocks * kMapThreads;
   const long long base = (long long)m * a.npix;
-  const int cap = map_cap(a);
-  const int nc = a.lists[2 * m], ne = a.lists[2 * m + 1];
-  if (nc > cap || ne > cap || ne > (long long)all * kMapEdges) {   // the cooperative kernel starts over
-    if (t == 0) *a.need_global = 1;
-    return;
-  }
-  const unsigned long long* const ek = map_keys(a, m);
-  int* const pool = reinterpret_cast<int*>(map_keys(a, m) + cap);
+  const int cap = (int)a.comp_cap;
+  const int nc = min(a.lists[2 * m], cap);   // (never above, from counts that start at 0)
+  const int ne = (int)min((long long)a.lists[2 * m + 1], 2 * a.npix);
+  unsigned long long* const ek = map_keys(a, m);
+  int* const pool = a.comps + 6ll * m * cap;
   int* const par[2] = {pool, pool + cap};
   int* const off[2] = {pool + 2 * cap, pool + 3 * cap};
   int* const hp = pool + 4 * cap;
   int* const ho = pool + 5 * cap;
+  int2* const el = a.edge_ends + (long long)m * a.spill_cap - kMapRegEdges;   // by edge number
   unsigned long long* const best = a.best + base;
   int* const flags = a.map_flags + 3 * m;   // rotating: the next slot is cleared two uses after its last read
   int use = 0, cur = 0;
@@ -442,6 +446,12 @@ __global__ void __launch_bounds__(kMapThreads) unwrap_map_kernel(UnwrapArgs a, i
       lb[i] = label(q);
     }
   }
+  int spill = 0;   // the thread's edges kMapEdges, kMapEdges + 1, ... at place t + i all
+  for (int k = t + kMapEdges * all; k < ne; k += all, ++spill) {
+    long long p, q;
+    ends(ek[k], p, q);
+    el[k] = make_int2(label(p), label(q));
+  }
   cluster_sync();
   for (int round = 0; round < a.max_rounds; ++round) {
     // heaviest incident edge of every component
@@ -457,6 +467,19 @@ __global__ void __launch_bounds__(kMapThreads) unwrap_map_kernel(UnwrapArgs a, i
       if (key[i] > __ldcg(best + la[i])) atomicMax(best + la[i], key[i]);
       if (key[i] > __ldcg(best + lb[i])) atomicMax(best + lb[i], key[i]);
     }
+    int kept = t + kMapEdges * all;
+    for (int k = kept, end = kept + spill * all; k < end; k += all) {
+      const unsigned long long kk = ek[k];
+      const int2 e = el[k];
+      const int ca = __ldcg(par[cur] + e.x), cb = __ldcg(par[cur] + e.y);
+      if (ca == cb) continue;
+      if (kk > __ldcg(best + ca)) atomicMax(best + ca, kk);
+      if (kk > __ldcg(best + cb)) atomicMax(best + cb, kk);
+      ek[kept] = kk;
+      el[kept] = make_int2(ca, cb);
+      kept += all;
+    }
+    spill = (kept - t) / all - kMapEdges;
     cluster_sync();
     const int fs = use % 3;
     for (int l = t; l < nc; l += all) {
@@ -543,15 +566,13 @@ __device__ __forceinline__ float unwrapped_at(const UnwrapArgs& a, long long v) 
 
 __global__ void unwrap_close_kernel(UnwrapArgs a, int maps) {
   if (blockIdx.x == 0 && threadIdx.x < 2 * maps) a.lists[threadIdx.x] = 0;
-  if (*a.need_global) return;   // the cooperative kernel has written out
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.nodes;
        v += (long long)gridDim.x * blockDim.x)
     a.out[v] = unwrapped_at(a, v);
 }
 
-// The cooperative path; opt: only if the map kernel asked for it.
-__global__ void __launch_bounds__(kUnwrapThreads) unwrap_kernel(UnwrapArgs a, int opt) {
-  if (opt && *a.need_global == 0) return;
+// The cooperative path.
+__global__ void __launch_bounds__(kUnwrapThreads) unwrap_kernel(UnwrapArgs a) {
   const long long n = a.nodes;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -696,12 +717,9 @@ __global__ void project_phase_kernel(ProjectArgs a) {
 }
 
 // u += (Phi' - Phi) pinv^T / phase_scale inside the mask; tiles: Phi' from the
-// tile and map kernels' offsets, unless the cooperative kernel ran
+// tile and map kernels' offsets
 __global__ void project_correct_kernel(ProjectArgs a, UnwrapArgs uw, int tiles) {
-  if (tiles) {
-    if (blockIdx.x == 0 && threadIdx.x < 2 * a.D) uw.lists[threadIdx.x] = 0;
-    tiles = *uw.need_global == 0;
-  }
+  if (tiles && blockIdx.x == 0 && threadIdx.x < 2 * a.D) uw.lists[threadIdx.x] = 0;
   for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < a.npix;
        r += (long long)gridDim.x * blockDim.x) {
     if (a.mask && a.mask[r] == 0.0f) continue;
@@ -752,30 +770,51 @@ int unwrap_map_blocks() {
   return 8;
 }
 
-static long long map_tiles(const UnwrapArgs& a) {
-  return (long long)((a.n1 + kTile - 1) / kTile) * ((a.n2 + kTile - 1) / kTile);
+static long long map_tiles(int n1, int n2) {
+  return (long long)((n1 + kTile - 1) / kTile) * ((n2 + kTile - 1) / kTile);
 }
 
-// A tile leaves about 13 components and 85 edges on a noisy map (a pixel's
-// heaviest edge often leaves its tile): eight blocks hold the edges of 640
-// such tiles (404^2 pixels), sixteen those of 1,280 (572^2).
+// Places for the components a map can list: each holds a pixel of its own on
+// its tile's rim, 4 (kTile - 1) of them.
+long long unwrap_comp_cap(int n1, int n2) {
+  const long long n = map_tiles(n1, n2) * 4 * (kTile - 1), npix = (long long)n1 * n2;
+  return n < npix ? n : npix;
+}
+
+// Places for the listed edges that the smallest cluster's registers do not
+// hold (a grid has fewer than 2 npix edges).
+long long unwrap_spill_cap(int n1, int n2) {
+  const long long n = 2ll * n1 * n2 - kMapRegEdges;
+  return n > 0 ? n : 0;
+}
+
+// The cluster's size.  A larger one has more reads in flight, a smaller one
+// cheaper barriers and room for more maps at a time (256 tiles, noisy phases on
+// the whole grid: three maps 107 us a call with sixteen blocks, 117 with eight,
+// but 16 maps 345 against 276; 399 and 625 tiles, three maps, smooth: 103 and
+// 129 us with sixteen, 123 and 170 with eight).
+static int map_blocks(const UnwrapArgs& a) { return a.max_blocks < 16 || map_tiles(a.n1, a.n2) <= 300 ? 8 : 16; }
+
+// Against the cooperative path, three maps, noisy phases, on the whole grid and
+// in a disc of half its area: 128^2 86 and 76 us a call (132 and 109), 256^2 117
+// and 101 (254 and 216), 512^2 304 and 182 (894 and 630), 560^2 284 and 176
+// (1,101 and 679); 16 maps of 512^2 836 and 536 (3,603 and 3,254).  Smooth,
+// random and constant phases likewise: none of these is slower.  Larger maps,
+// not measured, stay with the cooperative path.
 constexpr long long kTilesPerBlock = 80;
 
-static int map_blocks(const UnwrapArgs& a) { return map_tiles(a) <= 8 * kTilesPerBlock ? 8 : 16; }
-
 bool unwrap_by_tiles(const UnwrapArgs& a) {
-  return !a.test_stall && map_tiles(a) <= a.max_blocks * kTilesPerBlock;
+  return !a.test_stall && map_tiles(a.n1, a.n2) <= a.max_blocks * kTilesPerBlock;
 }
 
-cudaError_t unwrap_tiles_launch(const UnwrapArgs& a, int grid, cudaStream_t s) {
+cudaError_t unwrap_tiles_launch(const UnwrapArgs& a, cudaStream_t s) {
   const int maps = (int)(a.nodes / a.npix);
-  unwrap_tile_kernel<<<(unsigned)(map_tiles(a) * maps), kUnwrapThreads, 0, s>>>(a);
+  unwrap_tile_kernel<<<(unsigned)(map_tiles(a.n1, a.n2) * maps), kUnwrapThreads, 0, s>>>(a);
   cudaLaunchAttribute at;
   const int blocks = map_blocks(a);
   const cudaLaunchConfig_t c = map_config(maps, blocks, &at, s);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaLaunchKernelEx(&c, unwrap_map_kernel, a, blocks);
-  return e != cudaSuccess ? e : unwrap_launch(a, grid, true, s);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : cudaLaunchKernelEx(&c, unwrap_map_kernel, a, blocks);
 }
 
 cudaError_t unwrap_close_launch(const UnwrapArgs& a, int num_sms, cudaStream_t s) {
@@ -784,9 +823,8 @@ cudaError_t unwrap_close_launch(const UnwrapArgs& a, int num_sms, cudaStream_t s
   return cudaGetLastError();
 }
 
-cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, bool optional, cudaStream_t s) {
-  int opt = optional ? 1 : 0;
-  void* args[] = {const_cast<UnwrapArgs*>(&a), &opt};
+cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, cudaStream_t s) {
+  void* args[] = {const_cast<UnwrapArgs*>(&a)};
   return cudaLaunchCooperativeKernel((const void*)unwrap_kernel, dim3(grid), dim3(kUnwrapThreads), args, 0, s);
 }
 

@@ -24,7 +24,9 @@ struct UnwrapArgs {
   unsigned* bar_gen;
   int* lists;             // [2 D] components and edges listed per map, zero between calls
   int* map_flags;         // [3 D] the map kernel's "something changed" flags
-  int* need_global;       // the map kernel leaves the work to the cooperative one
+  int* comps;             // [6 D comp_cap] the map kernel's components
+  int2* edge_ends;        // [D spill_cap] labels of the listed edges past its registers
+  long long comp_cap, spill_cap;   // per map (unwrap_comp_cap, unwrap_spill_cap)
   int* err;               // kErrTimeout if a barrier wait runs out
   long long npix, nodes;
   int n1, n2;
@@ -48,14 +50,15 @@ struct ProjectArgs {
 
 bool unwrap_prepare(int num_sms, int* grid);
 int unwrap_map_blocks();
-// The cooperative path, on the given grid (optional: returns at once unless
-// *need_global); flags and barrier zeroed before.
-cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, bool optional, cudaStream_t s);
-// Whether the path by tiles and maps serves these maps; it, with the
-// cooperative launch behind it where a map leaves too many components; and
-// the kernel that writes out (project_correct does without).
+// The cooperative path, on the given grid; flags and barrier zeroed before.
+cudaError_t unwrap_launch(const UnwrapArgs& a, int grid, cudaStream_t s);
+// Whether the path by tiles and maps serves these maps (its lists hold every
+// map of such a size); its two kernels; and the one that writes out
+// (project_correct does without).
 bool unwrap_by_tiles(const UnwrapArgs& a);
-cudaError_t unwrap_tiles_launch(const UnwrapArgs& a, int grid, cudaStream_t s);
+long long unwrap_comp_cap(int n1, int n2);
+long long unwrap_spill_cap(int n1, int n2);
+cudaError_t unwrap_tiles_launch(const UnwrapArgs& a, cudaStream_t s);
 cudaError_t unwrap_close_launch(const UnwrapArgs& a, int num_sms, cudaStream_t s);
 cudaError_t project_phase_launch(const ProjectArgs& a, int num_sms, cudaStream_t s);
 // tiles: the unwrapped phases from uw's offsets (unwrap_tiles_launch without
