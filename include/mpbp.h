@@ -106,12 +106,11 @@ typedef struct {
                                  (both at most: the deterministic mode clears
                                  its pieces only where frames leave gaps)     */
   int32_t precision;          /* MPBP_PRECISION_* of the gradient evaluations */
-  int32_t tile_copies;        /* FFT kernels that take their inputs by TMA tile and
-                                 bulk copies of unpadded rows: bit 0 the gradient
-                                 kernel, bit 1 the forward kernel (none when a row
-                                 of n2 values is not a multiple of 16 bytes, i.e.
-                                 odd n2: the context then keeps O in rows of
-                                 n2 + 1, and the tile copies read those)       */
+  int32_t tile_copies;        /* FFT kernels that read rows of n2 values of O by
+                                 TMA tile copies: bit 0 the gradient kernel, bit 1
+                                 the forward kernel.  0 for odd n2, where O has
+                                 rows of n2 + 1; mpbp_input_copies tells what a
+                                 context's kernels use in either case          */
   int32_t fft_schedule;       /* MPBP_FFT_* in use (frame side 128)            */
   int32_t deterministic;      /* 1: the gradient sums are bitwise reproducible
                                  (mpbp_set_deterministic)                     */
@@ -436,8 +435,9 @@ mpbp_status mpbp_set_fft_schedule(mpbp_ctx *ctx, int32_t schedule);
  * on a 1024^2 object; 8 x 64 x (rows + 64) at side 64),
  * allocated here and kept while the context lives, and the clearing and
  * summing of it on each evaluation.  Needs frame side 64 or 128 on FP32 FFTs
- * (at 128 the exchange schedule) and rows of n2 values that are a multiple of
- * 16 bytes (even n2): else MPBP_ERR_UNSUPPORTED.  While on, evaluations over a frame list
+ * (at 128 the exchange schedule), tile copies and even n2: else
+ * MPBP_ERR_UNSUPPORTED.  (Odd n2 was refused when it had no tile copies; it has
+ * them now, and stays refused because nothing has asked for it.)  While on, evaluations over a frame list
  * (mpbp_loss_grad with frames, mpbp_adam_step minibatches), the host-buffer
  * calls, mpbp_loss_grad_batched and mpbp_autotune return
  * MPBP_ERR_UNSUPPORTED, and so do mpbp_set_precision / mpbp_set_fft_schedule
@@ -486,6 +486,20 @@ mpbp_status mpbp_set_precision(mpbp_ctx *ctx, int32_t mode);
  * while it is on are meaningless.  No effect on contexts whose frame kernels
  * use cp.async copies (M <= 16).  Off by default. */
 mpbp_status mpbp_set_test_stall(mpbp_ctx *ctx, int32_t on);
+
+/* How the context's FP32 FFT kernels take their inputs now, the gradient (and
+ * loss) kernel and the forward kernel, one of MPBP_COPIES_*. */
+#define MPBP_COPIES_ELEMENT 0     /* per-element cp.async                       */
+#define MPBP_COPIES_TILE 1        /* TMA tile and bulk copies                   */
+#define MPBP_COPIES_TILE_PADDED 2 /* the same, O in rows of n2 + 1 (odd n2)     */
+mpbp_status mpbp_input_copies(const mpbp_ctx *ctx, int32_t *gradient, int32_t *forward);
+
+/* Test support: with on != 0 the context's kernels take their inputs by
+ * per-element cp.async copies, as on a system whose driver encodes no tensor
+ * map; with 0 (the default) as mpbp_create chose.  Holds for what is enqueued
+ * afterwards (a captured step keeps its copies).  MPBP_ERR_UNSUPPORTED while
+ * the deterministic gradient is on, which needs tile copies. */
+mpbp_status mpbp_set_test_element_copies(mpbp_ctx *ctx, int32_t on);
 
 /* Turns on (enable != 0) or off the recording of CUDA events around every
  * launch of the fused frame kernel, on the stream it is launched on.  Off by

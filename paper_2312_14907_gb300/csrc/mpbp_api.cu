@@ -40,7 +40,8 @@ struct mpbp_ctx {
   FrameKernelInfo fk_fft{};   // the FFT kernels (forward mode always uses them)
   // tensor maps of O for the FFT kernels' tile copies (box widths from fk_fft)
   TmaMap tm_grad{}, tm_fwd{};
-  bool tile_grad = false, tile_fwd = false;
+  bool tile_grad = false, tile_fwd = false;           // tile copies in use ...
+  bool tile_grad_map = false, tile_fwd_map = false;   // ... and available (mpbp_set_test_element_copies)
   unsigned test_tx_extra = 0;   // mpbp_set_test_stall
   // host path: tensor maps of the staged counts, one per staging slot
   CUtensorMap ymap[kStageSlots];
@@ -721,8 +722,8 @@ mpbp_status mpbp_create(const mpbp_problem* pr, mpbp_ctx** out) {
   c->g_alpha_base = reinterpret_cast<double*>(b + oGAB);
   c->err = reinterpret_cast<int*>(b + oErr);
   c->arrivals = reinterpret_cast<unsigned*>(b + oArr);
-  c->tile_grad = encode_objects_map(c, c->fk_fft.tile_w_grad, &c->tm_grad);
-  c->tile_fwd = encode_objects_map(c, c->fk_fft.tile_w_fwd, &c->tm_fwd);
+  c->tile_grad = c->tile_grad_map = encode_objects_map(c, c->fk_fft.tile_w_grad, &c->tm_grad);
+  c->tile_fwd = c->tile_fwd_map = encode_objects_map(c, c->fk_fft.tile_w_fwd, &c->tm_fwd);
 
   std::vector<int2> sc(c->J);
   for (int j = 0; j < c->J; ++j) sc[j] = make_int2(pr->scan[2 * j], pr->scan[2 * j + 1]);
@@ -800,7 +801,7 @@ mpbp_status mpbp_get_info(const mpbp_ctx* c, mpbp_info* info) {
   info->launches_loss_grad = c->det ? 5 : 3;
   info->launches_step = c->det ? 5 : 3;
   info->precision = c->precision;
-  // odd n2: by tile copies of padded rows, which the flags do not count
+  // rows of n2 values only (mpbp_input_copies: what is in use for odd n2 too)
   info->tile_copies = (c->n2 & 1) ? 0 : (c->tile_grad ? 1 : 0) | (c->tile_fwd ? 2 : 0);
   info->fft_schedule = c->fft_schedule;
   info->deterministic = c->det ? 1 : 0;
@@ -817,8 +818,9 @@ mpbp_status mpbp_set_deterministic(mpbp_ctx* c, int32_t on) {
     return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs frame side 64 or 128");
   if (c->precision != MPBP_PRECISION_FP32 || (c->M == 128 && c->fft_schedule != kLayoutExchange))
     return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs FP32 FFTs (at 128: the exchange schedule)");
+  // odd n2: no kernel needs it refused any more, but the answer stays what it was
   if (!c->tile_grad || (c->n2 & 1))
-    return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs even n2 (rows of n2 values a multiple of 16 bytes)");
+    return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs tile copies and even n2");
   const mpbp_status r = det_prepare(c, frames_grid_for(c, c->nframes));
   if (r != MPBP_OK) return r;
   c->det = true;
@@ -2154,6 +2156,23 @@ mpbp_status mpbp_set_test_stall(mpbp_ctx* c, int32_t on) {
   if (!c) return MPBP_ERR_INVALID_ARG;
   c->test_tx_extra = on ? 16u : 0u;
   c->version++;   // batched plans copy the tensor maps with the hook
+  return MPBP_OK;
+}
+
+mpbp_status mpbp_input_copies(const mpbp_ctx* c, int32_t* gradient, int32_t* forward) {
+  if (!c || !gradient || !forward) return MPBP_ERR_INVALID_ARG;
+  const int32_t tile = (c->n2 & 1) ? MPBP_COPIES_TILE_PADDED : MPBP_COPIES_TILE;
+  *gradient = c->tile_grad ? tile : MPBP_COPIES_ELEMENT;
+  *forward = c->tile_fwd ? tile : MPBP_COPIES_ELEMENT;
+  return MPBP_OK;
+}
+
+mpbp_status mpbp_set_test_element_copies(mpbp_ctx* c, int32_t on) {
+  if (!c) return MPBP_ERR_INVALID_ARG;
+  if (c->det && on) return fail(c, MPBP_ERR_UNSUPPORTED, "the deterministic gradient needs tile copies");
+  c->tile_grad = !on && c->tile_grad_map;
+  c->tile_fwd = !on && c->tile_fwd_map;
+  c->version++;   // batched plans follow the copies
   return MPBP_OK;
 }
 

@@ -84,7 +84,11 @@ EXPORTS = ["mpbp_status_string", "mpbp_create", "mpbp_destroy", "mpbp_last_error
            "mpbp_loss_grad_phases", "mpbp_unwrap_phases", "mpbp_project_displacement",
            "mpbp_illumination", "mpbp_set_test_stall", "mpbp_loss_grad_host_counts16",
            "mpbp_set_scan_offsets", "mpbp_shift_probe", "mpbp_loss", "mpbp_set_fft_schedule",
-           "mpbp_set_deterministic"]
+           "mpbp_set_deterministic", "mpbp_input_copies", "mpbp_set_test_element_copies"]
+
+COPIES_ELEMENT = 0        # how a kernel's inputs arrive (Problem.input_copies): per-element cp.async,
+COPIES_TILE = 1           # TMA tile and bulk copies,
+COPIES_TILE_PADDED = 2    # the same, the objects in rows of n2 + 1 (odd n2)
 
 FFT_SHUFFLE = 0           # M = 128: radix-2 stages across threads by warp shuffles
 FFT_EXCHANGE = 1          # M = 128: three register layouts joined by shared-memory exchanges
@@ -181,6 +185,10 @@ def load(build_if_missing=True):
     lib.mpbp_frames_timing.restype = st
     lib.mpbp_set_test_stall.argtypes = [V, I32]
     lib.mpbp_set_test_stall.restype = st
+    lib.mpbp_input_copies.argtypes = [V, P(I32), P(I32)]
+    lib.mpbp_input_copies.restype = st
+    lib.mpbp_set_test_element_copies.argtypes = [V, I32]
+    lib.mpbp_set_test_element_copies.restype = st
     lib.mpbp_frames_timing_read.argtypes = [V, P(D), P(I32)]
     lib.mpbp_frames_timing_read.restype = st
     lib.mpbp_loss_grad_noalloc.argtypes = [P(_Problem), V, V, V, V, V, V, V, V, V, V, V]
@@ -547,6 +555,16 @@ class Problem:
     def read_state(state):
         raw = state.cpu().numpy().tobytes()
         return StepState.from_buffer_copy(raw)
+
+    def input_copies(self):
+        """How the gradient and the forward kernel take their inputs (COPIES_*; mpbp_input_copies)."""
+        g, f = ctypes.c_int32(), ctypes.c_int32()
+        self._check(self._lib.mpbp_input_copies(self._h, ctypes.byref(g), ctypes.byref(f)), "mpbp_input_copies")
+        return g.value, f.value
+
+    def set_test_element_copies(self, on=True):
+        """Test support: inputs by per-element copies (mpbp_set_test_element_copies)."""
+        self._check(self._lib.mpbp_set_test_element_copies(self._h, int(bool(on))), "mpbp_set_test_element_copies")
 
     def set_test_stall(self, on=True):
         """Test hook: the tile-copy waits of the frame kernels run out (MPBP_ERR_TIMEOUT)."""
