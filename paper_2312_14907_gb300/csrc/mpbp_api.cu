@@ -503,6 +503,7 @@ ObjectArgs object_args(const mpbp_ctx* c, const float* rho, const float* u, cons
   oa.npix = c->npix;
   oa.n2 = c->n2;
   oa.pitch = out == c->O ? c->o_pitch : c->n2;   // a caller's buffer has rows of n2
+  oa.o_stride = (long long)c->n1 * oa.pitch;
   oa.D = c->D;
   oa.C = c->C;
   oa.pc = c->pc;

@@ -44,35 +44,43 @@ __device__ __forceinline__ ObjIn object_load(const ObjectArgs& a, long long p) {
   return in;
 }
 
-// block bid of the nblk that work on a
-template <int FORM>
+// Whether rows of O are longer than n2 (o_pitch), known where the launch is
+// built; the Adam form tests it (built for each, it takes 80 registers in place
+// of 55, and a step on a 2048^2 object 186 us in place of 179).
+enum ObjectRows { kRowsTight, kRowsPadded, kRowsTest };
+
+// Block bid of the nblk that work on a.  Each pixel's inputs are read while the one before is on its way out.  The
+// peaks' alpha come straight from global memory but in the Adam form, which
+// has to form them first (kept in shared memory behind a barrier, with the row
+// length divided out and tested per thread, the u form took 5.7 us for three
+// peaks of 512^2 and 11.4 for 1024^2; so it takes 5.0 and 10.3).
+template <int FORM, int ROWS>
 __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int nblk) {
   const long long stride = (long long)nblk * blockDim.x;
-  const int pad = a.pitch - a.n2;
-  const long long ostride = a.npix / a.n2 * a.pitch;
-  __shared__ float s_alpha[kMaxPeaks];
   // the first pixel's reads are in flight beside the peaks'
   long long p = (long long)bid * blockDim.x + threadIdx.x;
   ObjIn in{};
   if (p < a.npix) in = object_load<FORM>(a, p);
-  if (threadIdx.x < a.D) {
-    const int m = threadIdx.x;
-    if constexpr (FORM == kObjAdam) s_alpha[m] = m == 0 ? 1.0f : expf(a.ad.alpha_t[m]);
-    else s_alpha[m] = a.alpha[m];
-  }
-  if (FORM == kObjAdam && bid == 0) {
-    mpbp_adam_state* st = a.ad.st;
-    const long long t = (long long)((unsigned long long)st->t + 1ull);   // any stored count
-    __syncthreads();   // every thread has read the old count
-    if (threadIdx.x == 0) {
-      st->t = t;
-      st->bc1 = one_minus_pow(st->beta1, t);
+  const float* alpha = a.alpha;
+  if constexpr (FORM == kObjAdam) {
+    __shared__ float s_alpha[kMaxPeaks];
+    if (threadIdx.x < a.D) s_alpha[threadIdx.x] = threadIdx.x == 0 ? 1.0f : expf(a.ad.alpha_t[threadIdx.x]);
+    alpha = s_alpha;
+    if (bid == 0) {
+      mpbp_adam_state* st = a.ad.st;
+      const long long t = (long long)((unsigned long long)st->t + 1ull);   // any stored count
+      __syncthreads();   // every thread has read the old count
+      if (threadIdx.x == 0) {
+        st->t = t;
+        st->bc1 = one_minus_pow(st->beta1, t);
+      }
+      if (threadIdx.x == 32) st->bc2 = one_minus_pow(st->beta2, t);
     }
-    if (threadIdx.x == 32) st->bc2 = one_minus_pow(st->beta2, t);
+    __syncthreads();
   }
-  __syncthreads();
   while (p < a.npix) {
-    const long long q = pad ? p + (unsigned)p / (unsigned)a.n2 * (long long)pad : p;   // npix < 2^31
+    const bool pad = ROWS == kRowsTest ? a.pitch != a.n2 : ROWS == kRowsPadded;
+    const long long q = pad ? p + (unsigned)p / (unsigned)a.n2 : p;   // npix < 2^31
     const float r = FORM == kObjAdam ? in.mask * expf(in.r) : in.r;
 #pragma unroll
     for (int m = 0; m < kMaxPeaks; ++m) {
@@ -86,8 +94,8 @@ __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int n
           for (int c = 0; c < kMaxComp; ++c) arg = fmaf(a.pc.kpi[m][c], in.uc[c], arg);
           sincospif(arg, &sn, &cs);   // exp(i phi), phi = pi * arg
         }
-        const float amp = s_alpha[m] * r;
-        reinterpret_cast<float2*>(a.O)[m * ostride + q] = make_float2(amp * cs, amp * sn);
+        const float amp = alpha[m] * r;
+        reinterpret_cast<float2*>(a.O)[m * a.o_stride + q] = make_float2(amp * cs, amp * sn);
       }
     }
     p += stride;
@@ -95,9 +103,9 @@ __device__ __forceinline__ void object_build(const ObjectArgs& a, int bid, int n
   }
 }
 
-template <int FORM>
+template <int FORM, int ROWS>
 __global__ void object_build_kernel(const __grid_constant__ ObjectArgs a) {
-  object_build<FORM>(a, blockIdx.x, gridDim.x);
+  object_build<FORM, ROWS>(a, blockIdx.x, gridDim.x);
 }
 
 // Which of the n problems of a batched launch block b works on: block0[k] is
@@ -112,7 +120,7 @@ __device__ __forceinline__ int batch_problem(const int* block0, int n, int b) {
 // 512^2: 16 launches of 4 us each became one).
 __global__ void object_build_batch_kernel(const __grid_constant__ ObjectBatch b) {
   const int k = batch_problem(b.block0, b.n, blockIdx.x);
-  object_build<kObjU>(b.a[k], blockIdx.x - b.block0[k], b.block0[k + 1] - b.block0[k]);
+  object_build<kObjU, kRowsTest>(b.a[k], blockIdx.x - b.block0[k], b.block0[k + 1] - b.block0[k]);
 }
 
 // ----------------------------------------------------------------------------
@@ -404,7 +412,12 @@ __device__ __forceinline__ void finish(const FinishArgs& a, const ReduceArgs& ra
   __shared__ double wsum[NW][NQ];
   __shared__ double s_loss;
   __shared__ float s_w[2];
-  __shared__ float s_alpha[MP];
+  // alpha through shared memory, which keeps the loads of one pixel together
+  // (read at its use, the sum over 2048^2 pixels of one peak took 278 us in
+  // place of 110); but with 16 phases a pixel the reads at use are the faster
+  // (512^2: 69.0 us a call against 69.9)
+  constexpr bool kAlphaShared = FORM != kFinPhi || MP < kMaxPeaks;
+  __shared__ float s_alpha[kAlphaShared ? MP : 1];
   __shared__ int s_accept;
   __shared__ bool last;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -428,7 +441,7 @@ __device__ __forceinline__ void finish(const FinishArgs& a, const ReduceArgs& ra
   }
   PixelIn<FORM, MP> in;
   if (p0 < a.npix) pixel_load<FORM, MP>(a, p0, in);
-  if (threadIdx.x < a.D) {
+  if (kAlphaShared && threadIdx.x < a.D) {
     const int m = threadIdx.x;
     if constexpr (FORM == kFinAdam) s_alpha[m] = m == 0 ? 1.0f : expf(a.ad.alpha_t[m]);
     else s_alpha[m] = a.alpha[m];
@@ -454,7 +467,7 @@ __device__ __forceinline__ void finish(const FinishArgs& a, const ReduceArgs& ra
       s_w[1] = (float)(d.t_new * sv.w_u);
     }
   }
-  __syncthreads();
+  if constexpr (kAlphaShared) __syncthreads();
   if constexpr (STEP) {
     accept = s_accept != 0;
     wr = s_w[0];
@@ -481,7 +494,7 @@ __device__ __forceinline__ void finish(const FinishArgs& a, const ReduceArgs& ra
         acc[m * a.npix + p] = make_float2(0.f, 0.f);
         const float Tr = fmaf(cs, A.x, -sn * A.y);
         const float Ti = fmaf(cs, A.y, sn * A.x);
-        const float am = s_alpha[m];
+        const float am = kAlphaShared ? s_alpha[m] : a.alpha[m];
         gr = fmaf(am, Tr, gr);
         const float dphi = -am * r * Ti;
         if constexpr (FORM == kFinPhi) {
@@ -805,9 +818,11 @@ static int grid_for(long long n, int threads, int cap) {
 
 cudaError_t launch_object_build(const ObjectArgs& a, int num_sms, cudaStream_t s) {
   const int grid = grid_for(a.npix, 256, num_sms * 8);
-  if (a.ad.chi) object_build_kernel<kObjAdam><<<grid, 256, 0, s>>>(a);
-  else if (a.phi) object_build_kernel<kObjPhi><<<grid, 256, 0, s>>>(a);
-  else object_build_kernel<kObjU><<<grid, 256, 0, s>>>(a);
+  const bool pad = a.pitch != a.n2;
+  auto* k = pad ? object_build_kernel<kObjU, kRowsPadded> : object_build_kernel<kObjU, kRowsTight>;
+  if (a.ad.chi) k = object_build_kernel<kObjAdam, kRowsTest>;
+  else if (a.phi) k = pad ? object_build_kernel<kObjPhi, kRowsPadded> : object_build_kernel<kObjPhi, kRowsTight>;
+  k<<<grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -128,8 +128,9 @@ struct ObjectArgs {
   const float* u;
   const float* phi;     // per-peak phases [D][npix] in place of u (or nullptr)
   const float* alpha;
-  cf* O;                // [D][npix / n2][pitch]
+  cf* O;                // [D][n1][pitch]
   long long npix;
+  long long o_stride;   // n1 * pitch
   int n2, pitch;
   int D, C;
   PhaseCoef pc;

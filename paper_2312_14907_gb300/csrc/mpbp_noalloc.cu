@@ -130,6 +130,7 @@ extern "C" mpbp_status mpbp_loss_grad_noalloc(const mpbp_problem* pr, const floa
   oa.alpha = alpha;
   oa.O = O;
   oa.n2 = oa.pitch = pr->n2;
+  oa.o_stride = npix;
   oa.npix = npix;
   oa.D = pr->npeaks;
   oa.C = pr->ncomp;
