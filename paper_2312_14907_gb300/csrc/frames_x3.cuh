@@ -650,9 +650,11 @@ MPBP_DI double x3_run(const FrameArgs& p, const TmaMap* tm, int lo, int hi, X3Bl
       }
       // a probe of the next frame's own: on its way to L2 while this frame is
       // transformed (512^2, 5,043 shifted probes: 494 -> 454 us a call)
-      if (p.probe_stride < 0 && threadIdx.x == 0 && nxt.valid)
-        bulk_prefetch(frame_probe(p, nxt, M * M), M * M * (uint32_t)sizeof(cf));
-      __syncwarp();
+      if (p.probe_stride < 0) {
+        if (threadIdx.x == 0 && nxt.valid)
+          bulk_prefetch(frame_probe(p, nxt, M * M), M * M * (uint32_t)sizeof(cf));
+        __syncwarp();
+      }
     }
     x3_frame<TMA, LOSS, BG, DET, FWD>(p, b.r, cur, nxt, [&](float fl) { lsum += (double)fl; }, b.bs, tm, b.buf, b.abuf,
                                       b.tp, b.ta, tab, win);
