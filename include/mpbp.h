@@ -344,9 +344,11 @@ mpbp_status mpbp_illumination(mpbp_ctx *ctx, float *out, void *stream);
  * 1: down}), i.e. integration along the maximum spanning forest.  Each
  * connected region is then shifted by the multiple of 2 pi that gives its
  * lowest-numbered pixel its wrapped value; pixels off the mask keep theirs.
- * The first call allocates the unwrapper's workspace (~52 bytes per pixel
- * and map) and synchronises.  One cooperative launch; its grid barriers are
- * bounded in time (MPBP_ERR_TIMEOUT via mpbp_sync_status if one runs out). */
+ * The first call allocates the unwrapper's workspace (64 bytes per pixel and
+ * map, up to 86 for maps of at most 1,280 tiles of 16 x 16) and synchronises.
+ * Maps of at most 1,280 tiles: three launches, whose only waits are hardware
+ * cluster barriers.  Larger ones: one cooperative launch; its grid barriers
+ * are bounded in time (MPBP_ERR_TIMEOUT via mpbp_sync_status if one runs out). */
 mpbp_status mpbp_unwrap_phases(mpbp_ctx *ctx, const float *wrapped, const float *mask,
                                float *out, void *stream);
 
@@ -370,9 +372,12 @@ mpbp_status mpbp_loss_grad_phases(mpbp_ctx *ctx, const float *rho, const float *
                                   void *stream);
 
 /* Loss and gradient of n independent problems (frame sides may differ) in
- * one persistent launch of the fused frame kernel.  Each argument is a host
- * array of n per-problem pointers with the meaning of mpbp_loss_grad
- * (all frames of each problem). */
+ * the fused launches that mpbp_set_batch_schedule describes.  Each argument is
+ * a host array of n per-problem pointers with the meaning of mpbp_loss_grad
+ * (all frames of each problem).  Problems may share an output buffer; it then
+ * holds the last one's (their gradients are assembled one after the other).
+ * A bounded wait that runs out ends its block: mpbp_sync_status of every
+ * problem whose frames the block leaves out returns MPBP_ERR_TIMEOUT. */
 mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx *const *ctxs,
                                    const float *const *rho, const float *const *u,
                                    const float *const *alpha, double *const *loss,
@@ -433,8 +438,8 @@ mpbp_status mpbp_set_fft_schedule(mpbp_ctx *ctx, int32_t schedule);
  * device workspace of about 8 x 128 x (rows spanned by a strip + 128) bytes
  * per piece for frame side 128 (about 1 GB for 87,846 frames of 128 x 128
  * on a 1024^2 object; 8 x 64 x (rows + 64) at side 64),
- * allocated here and kept while the context lives, and the clearing and
- * summing of it on each evaluation.  Needs frame side 64 or 128 on FP32 FFTs
+ * allocated here and kept while the context lives, and on each evaluation its
+ * summing (and, where a strip's frames leave rows between them, its clearing).  Needs frame side 64 or 128 on FP32 FFTs
  * (at 128 the exchange schedule), tile copies and even n2: else
  * MPBP_ERR_UNSUPPORTED.  (Odd n2 was refused when it had no tile copies; it has
  * them now, and stays refused because nothing has asked for it.)  While on, evaluations over a frame list

@@ -194,6 +194,40 @@ bool batch_fused(int mode, const mpbp_ctx* c) {
   return c->M < 128 || mode == 0 || (mode == 1 && c->tile_grad);
 }
 
+// whether no output of a batched call overlaps another output or an input
+bool outputs_apart(int n, mpbp_ctx* const* ctxs, const float* const* rho, const float* const* u,
+                   const float* const* alpha, double* const* loss, float* const* g_rho, float* const* g_u,
+                   double* const* g_alpha) {
+  struct Span {
+    uintptr_t lo, hi;
+    bool out;
+  };
+  std::vector<Span> v;
+  v.reserve(7 * (size_t)n);
+  auto add = [&](const void* p, size_t bytes, bool out) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p);
+    if (a) v.push_back(Span{a, a + bytes, out});
+  };
+  for (int i = 0; i < n; ++i) {
+    const size_t np = sizeof(float) * (size_t)ctxs[i]->npix, nu = np * ctxs[i]->C, D = ctxs[i]->D;
+    add(rho[i], np, false);
+    add(u[i], nu, false);
+    add(alpha[i], sizeof(float) * D, false);
+    add(loss[i], sizeof(double), true);
+    add(g_rho[i], np, true);
+    add(g_u[i], nu, true);
+    if (g_alpha) add(g_alpha[i], sizeof(double) * D, true);
+  }
+  std::sort(v.begin(), v.end(), [](const Span& a, const Span& b) { return a.lo < b.lo; });
+  uintptr_t any = 0, out = 0;   // ends of the spans so far
+  for (const Span& s : v) {
+    if (s.lo < (s.out ? any : out)) return false;
+    any = std::max(any, s.hi);
+    if (s.out) out = std::max(out, s.hi);
+  }
+  return true;
+}
+
 // frame-range launches of one host-path evaluation (each writes its own
 // slice of the loss partials)
 constexpr int kMaxHostChunks = 8;
@@ -1919,11 +1953,14 @@ mpbp_status mpbp_loss_grad_batched(int32_t n, mpbp_ctx* const* ctxs, const float
     c->acc_dirty = true;
     MPBP_CUDA(c, launch_frames(c, fa, grid_of[i], s));
   }
-  // A6/A7 tail and A8 reductions of every problem
+  // A6/A7 tail and A8 reductions of every problem; one after the other where
+  // an output is shared (a caller after the losses alone may pass one scratch
+  // gradient for all), so that what stands there in the end is the last one's
   int k = 0;
-  for (int i0 = 0; i0 < n; i0 += kAuxBatch) {
+  const int step = outputs_apart(n, ctxs, rho, u, alpha, loss, g_rho, g_u, g_alpha) ? kAuxBatch : 1;
+  for (int i0 = 0; i0 < n; i0 += step) {
     FinishBatch fb;
-    fb.n = std::min(n - i0, kAuxBatch);
+    fb.n = std::min(n - i0, step);
     for (int j = 0; j < fb.n; ++j) {
       const int i = i0 + j;
       mpbp_ctx* c = ctxs[i];
