@@ -625,8 +625,9 @@ mpbp_status enqueue_loss_grad(mpbp_ctx* c, const float* rho, const float* u, con
 }
 
 // The six moment arrays; theirs: the caller's side of the copies.  One launch
-// where that side is device memory, else (not a use the interface names) the
-// runtime's copies and what they answer.
+// where that side is device memory and the copies' targets lie apart, else (not
+// a use the interface names) the runtime's copies, in this order, and what they
+// answer.
 mpbp_status copy_moments(mpbp_ctx* c, void* const* to, const void* const* from, const void* const* theirs,
                          cudaStream_t s) {
   const long long np = c->npix, nu = c->npix * c->C;
@@ -641,6 +642,8 @@ mpbp_status copy_moments(mpbp_ctx* c, void* const* to, const void* const* from, 
     a.dst[i] = static_cast<uint32_t*>(to[i]);
     a.src[i] = static_cast<const uint32_t*>(from[i]);
     a.words[i] = words[i];
+    for (int k = 0; k < i; ++k)
+      device = device && (a.dst[i] + words[i] <= a.dst[k] || a.dst[k] + words[k] <= a.dst[i]);
   }
   if (device) {
     MPBP_CUDA(c, launch_moment_copy(a, c->num_sms, s));
