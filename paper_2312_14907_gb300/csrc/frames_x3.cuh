@@ -153,9 +153,12 @@ struct X3Win {
 // converged; ta: the thread's lane at the window's first column.  With a
 // deterministic plan the rows go to the block's current piece instead:
 // rows outside the hull of those written so far are stored, the others
-// loaded, added and stored (the piece has no other writer, it starts
-// cleared, and successive write-backs of a row are separated by block
-// barriers); on a strip the window slides down, so every row is a store.
+// loaded, added and stored (the piece has no other writer, and successive
+// write-backs of a row are separated by block barriers); on a strip the
+// window slides down, so every row is a store.  A piece is not cleared
+// beforehand: its frames come in ascending rows, so that the hull grows at its
+// end alone and has no hole unless two of them are more than a frame apart,
+// and then the host clears the pieces first (mpbp_ctx::det_gaps).
 template <bool DET>
 MPBP_DI void x3_flush(const FrameArgs& p, const X3Roles& r, const X3Win& w, int x0, int d, uint32_t ta,
                       bool zero) {
